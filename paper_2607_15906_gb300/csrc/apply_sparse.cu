@@ -9,32 +9,41 @@
 //
 //  * a listing pass writes the nonzero amplitudes (index, value) in index
 //    order, and the first entry of every tile;
-//  * a block (one per SM) owns an output tile t of 2^LB amplitudes and
-//    accumulates it in shared memory.  Its work units are (piece, chunk):
-//    32 sp_amps consecutive nonzero amplitudes of the piece's source tile
-//    u = t ^ (x >> LB), sp_amps per lane, against the piece's groups, which
-//    the warp walks together.  Units are numbered piece by piece from a
-//    per-tile scan of chunk counts and claimed a few at a time.  For a group with mask x the lane's
-//    amplitude psi(k') goes to output k = k' ^ x with weight D(k): a LUT
-//    group reads its entry at code(k) (the code is linear in k over GF(2)),
-//    a term-list group sums its terms' signs at k (times the factor 0 or 2
-//    of a paired group).  A nonzero product is added to the accumulator, in
-//    64-bit fixed point, with shared-memory integer atomics; a zero weight
-//    adds nothing and is left out.  For complex128 a LUT group's nonzero
-//    (amplitude, weight) items are first packed into a per-warp buffer and
-//    multiplied and added 32 at a time, so that the FP64 products and
-//    conversions run with every lane busy (about two thirds of the items of
-//    a sector-confined state have a zero weight);
+//  * a block (one per SM) owns an output tile t of 2^kSpLB amplitudes and
+//    accumulates it in shared memory.  Its work units are (piece, span of
+//    chunks): 32 consecutive nonzero amplitudes, one per lane, of the piece's
+//    source tile u = t ^ (x >> kSpLB), against the piece's groups.  Units are
+//    numbered piece by piece from a per-tile scan and claimed by the warps;
+//  * the host splits every LUT group into cases (see SpHead): a case applies
+//    where up to three parities of the output index are zero.  A head of 32
+//    cases has its 4 x 32 parities from three 16-byte table reads, and the
+//    cases that apply to a lane's amplitude are one word, so a lane spends
+//    instructions only on nonzero products: about a sixth of the (amplitude,
+//    case) pairs of a sector-confined state.  Testing every (amplitude, group)
+//    pair by population counts, as before, took two thirds of the issue slots;
+//  * a case whose parities the tile's bits alone make one is dead in the whole
+//    tile; pieces with only dead cases get no units there (half of the units
+//    at 24 qubits, three fifths at 28);
+//  * term-list groups take their weight from tables over index ranges (SpTab),
+//    summed in integers; the diagonal group and the identity are units over
+//    the own tile's amplitudes;
+//  * a product is added to the accumulator, in fixed point, with shared-memory
+//    integer atomics.  A warp whose amplitudes are all real (every state of a
+//    real H and pool) forms no imaginary products;
 //  * after the last unit, lanes over the nonzero amplitudes of the own tile
-//    add the diagonal group and the identity and take the energy partials;
-//    then the whole tile (zeros included) is streamed to H psi.
+//    take the energy partials, and the whole tile (zeros included) is streamed
+//    to H psi.
 //
-// Every lane does the same work for every group, whatever the sparsity
-// pattern, and a group's descriptor and LUT are read at one address per
-// warp (from global memory through L1).  The order in which products reach
-// an accumulator element is not fixed, but integer addition does not depend
-// on it: H psi, E and everything computed from them are reproducible bit
-// for bit from run to run.
+// The order in which products reach an accumulator element is not fixed, but
+// integer addition does not depend on it: H psi, E and everything computed
+// from them are reproducible bit for bit from run to run.
+//
+// What bounds it (24 qubits, 233,867 nonzero amplitudes, 2.3e8 nonzero
+// products): instruction issue and the latency of the table reads, 54 % of the
+// issue slots busy with 7.2e8 warp instructions; the shared-memory atomics'
+// wavefronts take 0.37 ms.  2.29 -> 1.21 ms (complex64), 6.24 -> 2.0 ms
+// (complex128), 18.0 -> 10.4 ms at 28 qubits, against the kernel that tested
+// every pair.
 //
 // The kernel is launched with the staged one; each returns at once unless
 // the count of nonzero amplitudes selects it, so the choice needs no host
@@ -52,21 +61,10 @@ namespace gocp {
 namespace {
 
 constexpr int kAmpBlock = 256;   // listing passes: one amplitude word (4 octets) per thread
-constexpr uint32_t kUnitBatch = 4;   // scatter work units per claim
+constexpr uint32_t kUnitBatch = 4;   // scatter work units per claim, at most
 
-// Nonzero source amplitudes per lane per work unit: complex64 two, with
-// FP32 products added at once; complex128 one, with integer products of the
-// fixed-point weights and amplitudes, its LUT-group items compacted per warp
-// (see sp_lut_q).
-template <typename R>
-__host__ __device__ constexpr int sp_amps() { return sizeof(R) == 4 ? 2 : 1; }
-
-// One block of 1024 threads (64 registers) per SM in both precisions
-// (complex128 measured 6.3 ms per 24-qubit call at 1024 threads, 6.6 at
-// 768, 7.8 at 512).
-template <typename R>
-__host__ __device__ constexpr int sp_threads() { return 1024; }
-
+// One block of 1024 threads (64 registers) per SM in both precisions.
+constexpr int kSpThreads = 1024;
 
 template <typename R>
 __device__ __forceinline__ void load_octet(const C_t<R>* __restrict__ psi, uint32_t octet, C_t<R> (&v)[kAmpsH]) {
@@ -244,309 +242,289 @@ k_tile_offsets(const uint32_t* __restrict__ idx, const uint32_t* __restrict__ le
   off[u] = lo;
 }
 
-// The tile's accumulator holds component j (2i: real part, 2i + 1:
-// imaginary part of member i) of octet o at j kOct + (o ^ 4i): a warp's
-// atomics on one component spread over the banks by octet, two members of
-// one octet fall on different banks, and the epilogue's reads of one
-// component stay a permutation of 32 consecutive words.
-template <uint32_t kOct>
-__device__ __forceinline__ uint32_t acc_at(uint32_t k) {
-  const uint32_t i = k & 7u, o = (k >> 3) & (kOct - 1u);
-  return (2u * i) * kOct + (o ^ (i << 2));
-}
-
 // Fixed-point accumulation.  A product p is added as the integer
 // round(p 2^F) (the amplitudes are scaled by 2^F once, see below), so the
 // sum is exact integer arithmetic: the same in any order of the atomics,
 // and the result is bit-for-bit reproducible.  F is chosen per call so that
 // the sum of the magnitudes of all contributions to one output component --
-// at most hbound x 2 max(|Re psi|, |Im psi|) -- stays below 2^62: no partial
-// sum can overflow.  For complex64, F also keeps every off-diagonal product
-// below 2^30, so that it converts with a 32-bit instruction; its rounding,
+// at most hbound x 2 max(|Re psi|, |Im psi|) -- stays below 2^62 (complex64:
+// 2^46): no partial sum can overflow.  For complex64, F also keeps every
+// off-diagonal product below 2^30, so that it converts with a 32-bit
+// instruction; its rounding,
 // at most 2^-(F+1), is then about 1e-9 of the largest possible product, and
 // an entry of H psi collects it from at most a few thousand products.  For
 // complex128 the rounding is at most 2^-(F+1) with F near 62 - log2 of the
 // bound, far below the FP64 rounding of the products.
+//
+// The tile's accumulator is four planes of 32-bit words, one word per
+// amplitude of the tile: low and high half of the real part, low and high
+// half of the imaginary part.  An atomic's bank is then the amplitude's low
+// five bits whatever the half, so a warp's 32 scattered adds spread over all
+// 32 banks (64-bit words side by side would put the low halves on 16).
+constexpr uint32_t kPlane = 4u * kSpTile;                                 // bytes of a plane
+constexpr uint32_t kRe = 0u, kIm = 2u * kPlane;                           // low planes; the high plane follows each
+constexpr uint32_t kAccBytes = 4u * kPlane;
 
-// Adds v to the 64-bit accumulator word p as two 32-bit atomics: the low
-// word's, and the high word's plus the carry out of the low word, taken from
-// the old value that atomic returns.  The pair is exact modulo 2^64 in any
-// order of the atomics (measured faster than one 64-bit atomic).  complex128
-// adds its products this way; complex64 uses the split form (fx_add_split).
-__device__ __forceinline__ void fx_add(unsigned long long* p, long long v) {
-  uint32_t* w = reinterpret_cast<uint32_t*>(p);
-  const uint32_t lo = (uint32_t)(unsigned long long)v, hi = (uint32_t)((unsigned long long)v >> 32);
-  const uint32_t old = atomicAdd(w, lo);
-  atomicAdd(w + 1, hi + (uint32_t)(old + lo < old));
+__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+// Shared-memory adds by 32-bit address and a constant offset.
+template <uint32_t OFF>
+__device__ __forceinline__ void red_add(uint32_t at, uint32_t v) {
+  asm volatile("red.shared.add.u32 [%0+%2], %1;" ::"r"(at), "r"(v), "n"(OFF) : "memory");
+}
+template <uint32_t OFF>
+__device__ __forceinline__ uint32_t atom_add(uint32_t at, uint32_t v) {
+  uint32_t old;
+  asm volatile("atom.shared.add.u32 %0, [%1+%3], %2;" : "=r"(old) : "r"(at), "r"(v), "n"(OFF) : "memory");
+  return old;
+}
+
+// One 64-bit accumulator component at byte offset `at` of its low plane.
+__device__ __forceinline__ long long acc_get(const uint8_t* acc, uint32_t at) {
+  return (long long)(((unsigned long long)*reinterpret_cast<const uint32_t*>(acc + at + kPlane) << 32) |
+                     *reinterpret_cast<const uint32_t*>(acc + at));
+}
+__device__ __forceinline__ void acc_set(uint8_t* acc, uint32_t at, long long v) {
+  *reinterpret_cast<uint32_t*>(acc + at) = (uint32_t)(unsigned long long)v;
+  *reinterpret_cast<uint32_t*>(acc + at + kPlane) = (uint32_t)((unsigned long long)v >> 32);
+}
+
+// Adds v to the component PL (kRe, kIm) of the amplitude at shared address at.
+//
+// Carry form (complex128): the low word's add, and the high word's plus the
+// carry out of the low word, taken from the old value that atomic returns;
+// exact modulo 2^64 in any order of the atomics (measured faster than one
+// 64-bit atomic).
+//
+// Split form (complex64, products below 2^30): the low plane sums the low 16
+// bits of each product (0 .. 65535) and the high plane the product shifted
+// right by 16 (arithmetic, |.| <= 2^14), two independent adds with no carry
+// between them.  With fewer than 65536 products per word (one per
+// off-diagonal group, and the diagonal's) the low half cannot wrap,
+// low < 2^16 * 65536 = 2^32, and the high half holds the word's total above
+// bit 16, |high| < 2^31.  The value is high * 2^16 + low, formed exactly once every
+// product has been added.
+template <bool SPLIT, uint32_t PL>
+__device__ __forceinline__ void fx_put(uint32_t at, long long v) {
+  const uint32_t lo = (uint32_t)(unsigned long long)v;
+  if constexpr (SPLIT) {
+    red_add<PL>(at, lo & 0xFFFFu);
+    red_add<PL + kPlane>(at, (uint32_t)((int)lo >> 16));
+  } else {
+    const uint32_t old = atom_add<PL>(at, lo);
+    red_add<PL + kPlane>(at, (uint32_t)((unsigned long long)v >> 32) + (uint32_t)(old + lo < old));
+  }
+}
+
+// A product of more than 32 bits (the diagonal's).  In split form: its low 16
+// bits into the low plane, the bits above into the high plane modulo 2^32;
+// only the word's total has to fit there, and it is below 2^46 by the choice
+// of F.
+template <bool SPLIT, uint32_t PL>
+__device__ __forceinline__ void fx_put_wide(uint32_t at, long long v) {
+  if constexpr (SPLIT) {
+    red_add<PL>(at, (uint32_t)v & 0xFFFFu);
+    red_add<PL + kPlane>(at, (uint32_t)(unsigned long long)(v >> 16));
+  } else {
+    fx_put<false, PL>(at, v);
+  }
 }
 
 // A scaled product as an integer.  complex64: every off-diagonal product is
 // below 2^30 by the choice of F, so a 32-bit conversion suffices (the 64-bit
-// conversions run on the FP64 pipe, narrow on this part); complex128: FP64
-// products, a 64-bit conversion.
-template <typename R>
-__device__ __forceinline__ long long fx_prod(R v) {
-  return sizeof(R) == 4 ? (long long)__float2int_rn((float)v) : __double2ll_rn((double)v);
-}
-
-// A scaled value up to 2^62 (the diagonal's products, once per amplitude).
-template <typename R>
-__device__ __forceinline__ long long fx_wide(R v) {
-  return sizeof(R) == 4 ? __float2ll_rn((float)v) : __double2ll_rn((double)v);
-}
+// conversions run on the FP64 pipe, narrow on this part).
+__device__ __forceinline__ long long fx_prod(float v) { return (long long)__float2int_rn(v); }
 
 // An accumulator value back in R (zeros, most of a sector state's tile,
 // skip the conversion).
 template <typename R>
-__device__ __forceinline__ R fx_val(unsigned long long a) {
-  if (a == 0ull) return R(0);
-  return sizeof(R) == 4 ? (R)__ll2float_rn((long long)a) : (R)__ll2double_rn((long long)a);
-}
-
-// Split form of the accumulator word (complex64, products below 2^30): its
-// low 32-bit half sums the low 16 bits of each product (0 .. 65535) and its
-// high half the product shifted right by 16 (arithmetic, |.| <= 2^14), two
-// independent atomics with no carry between them.  With fewer than 65536
-// products per word (one per off-diagonal group) neither half can wrap:
-// low < 2^16 * 65536 = 2^32, |high| < 2^30.  The word's value is
-// high * 2^16 + low, formed exactly by split_to_wide once every product has
-// been added.
-__device__ __forceinline__ void fx_add_split(unsigned long long* p, int v) {
-  uint32_t* w = reinterpret_cast<uint32_t*>(p);
-  atomicAdd(w, (uint32_t)v & 0xFFFFu);
-  atomicAdd(w + 1, (uint32_t)(v >> 16));
-}
-
-__device__ __forceinline__ unsigned long long split_to_wide(unsigned long long w) {
-  const long long high = (long long)(int)(uint32_t)(w >> 32);
-  return (unsigned long long)(high * 65536ll + (long long)(w & 0xffffffffull));
-}
-
-template <uint32_t kOct, bool SPLIT = false>
-__device__ __forceinline__ void acc_add(unsigned long long* acc, uint32_t k, long long re, long long im) {
-  const uint32_t at = acc_at<kOct>(k);
-  if constexpr (SPLIT) {
-    fx_add_split(acc + at, (int)re);
-    fx_add_split(acc + at + kOct, (int)im);
-  } else {
-    fx_add(acc + at, re);
-    fx_add(acc + at + kOct, im);
-  }
-}
-
-// One LUT group (descriptor in global memory, read through L1 at one
-// address per warp) against the lane's nonzero amplitudes psi(ks[s]), whose
-// values vs[s] are pre-scaled by 2^F.  The entry's magnitude depends on
-// phi(k) alone (lut16[phi | 8] = -lut16[phi]), so the sign parity is taken
-// only for a nonzero entry.
-template <typename R, uint32_t kOct, int A, bool SPLIT>
-__device__ __forceinline__ void sp_lut(const HLut<R>* __restrict__ L, const uint4 h0, const uint32_t v2,
-                                       const uint32_t (&ks)[A], const C_t<R> (&vs)[A], const bool (&valid)[A],
-                                       unsigned long long* acc) {
-#pragma unroll
-  for (int s = 0; s < A; ++s) {
-    const uint32_t k = ks[s] ^ h0.x;
-    const uint32_t phi = (uint32_t)(__popc(k & h0.z) & 1) | ((uint32_t)(__popc(k & h0.w) & 1) << 1) |
-                         ((uint32_t)(__popc(k & v2) & 1) << 2);
-    const R d0 = __ldg(L->lut16 + phi);
-    if (valid[s] && d0 != R(0)) {
-      const R d = (__popc(k & h0.y) & 1) ? -d0 : d0;
-      acc_add<kOct, SPLIT>(acc, k, fx_prod<R>(d * vs[s].x), fx_prod<R>(d * vs[s].y));
-    }
-  }
+__device__ __forceinline__ R fx_val(long long a) {
+  if (a == 0ll) return R(0);
+  return sizeof(R) == 4 ? (R)__ll2float_rn(a) : (R)__ll2double_rn(a);
 }
 
 // complex128 products in integers.  The weights (LUT entries and term-list
-// weights) are stored as d_q = round(d 2^Fd) (DevTables::twfix, |d_q| < 2^62)
-// and the lane's amplitude components as v_q = round(v 2^(F + 63 - Fd))
-// (|v_q| < 2^63: |v| 2^F < 2^61 / hbound and hbound >= dmax >= 2^(61 - Fd));
-// their product shifted right by 63 is round(d v 2^F), the fixed-point
-// product, formed exactly and rounded once.  FP64 instructions run on a pipe
-// about 1/64 the width of FP32 here; these are integer instructions.
+// weights) are stored as d_q = round(d 2^Fd) (|d_q| < 2^62) and the lane's
+// amplitude components as v_q = round(v 2^(F + 63 - Fd)) (|v_q| < 2^63:
+// |v| 2^F < 2^61 / hbound and hbound >= dmax >= 2^(61 - Fd)); their product
+// shifted right by 63 is round(d v 2^F), the fixed-point product, formed
+// exactly and rounded once.  FP64 instructions run on a pipe about 1/64 the
+// width of FP32 here; these are integer instructions.
 __device__ __forceinline__ long long q_mul(long long a, long long b) {
   const unsigned long long hi = (unsigned long long)__mul64hi(a, b);
   const unsigned long long lo = (unsigned long long)a * (unsigned long long)b;
   return (long long)((hi << 1) + (lo >> 63) + ((lo >> 62) & 1ull));
 }
 
-// A compacted complex128 item: the output index k, the weight d_q and the
-// lane's amplitude v_q.  A warp's buffer holds up to 32 (A + 1) items: at
-// most 31 wait after a flush and a group adds at most 32 A.
-struct __align__(16) SpItemQ {
-  uint32_t k, pad;
-  long long d, vx, vy;
-};
-constexpr uint32_t kSpCapQ = 32u * (uint32_t)(sp_amps<double>() + 1);
+// The lane's amplitude in the form its products take: scaled by 2^F
+// (complex64), or as v_q (complex128, see q_mul).
+template <typename R> struct SpVal;
+template <> struct SpVal<float> { using T = float; };
+template <> struct SpVal<double> { using T = long long; };
 
-// Adds buffered item `at` (if `on`) to the accumulator; the warp
-// synchronises before (the items are other lanes' stores) and after (the
-// slots are then reused).
-template <uint32_t kOct>
-__device__ __forceinline__ void sp_flush_q(const SpItemQ* wb, uint32_t at, bool on, unsigned long long* acc) {
-  __syncwarp();
-  if (on) {
-    const SpItemQ e = wb[at];
-    acc_add<kOct>(acc, e.k, q_mul(e.d, e.vx), q_mul(e.d, e.vy));
-  }
-  __syncwarp();
+__device__ __forceinline__ long long sp_product(float d, float v) { return fx_prod(d * v); }
+__device__ __forceinline__ long long sp_product(long long d, long long v) { return q_mul(d, v); }
+
+// d negated by the top bit of s.
+__device__ __forceinline__ float sp_signed(float d, uint32_t s) {
+  return __uint_as_float(__float_as_uint(d) ^ (s & 0x80000000u));
+}
+__device__ __forceinline__ long long sp_signed(long long d, uint32_t s) {
+  const long long m = (long long)((int)s >> 31);
+  return (d ^ m) - m;
 }
 
-// complex128 LUT group: the integer LUT entry lq[phi] (the group's lut16 in
-// the fixed-point copy of the blob), nonzero items appended to the warp's
-// buffer (cnt items, warp-uniform) in lane order; lt = the lanes below this
-// one.  About two thirds of a sector-confined state's items have a zero
-// weight, so the products run 32 at a time with every lane busy.
-template <uint32_t kOct, int A>
-__device__ __forceinline__ void sp_lut_q(const long long* __restrict__ lq, const uint4 h0, const uint32_t v2,
-                                         const uint32_t (&ks)[A], const long long (&vx)[A],
-                                         const long long (&vy)[A], const bool (&valid)[A], SpItemQ* wb,
-                                         uint32_t& cnt, const uint32_t lt) {
-#pragma unroll
-  for (int s = 0; s < A; ++s) {
-    const uint32_t k = ks[s] ^ h0.x;
-    const uint32_t phi = (uint32_t)(__popc(k & h0.z) & 1) | ((uint32_t)(__popc(k & h0.w) & 1) << 1) |
-                         ((uint32_t)(__popc(k & v2) & 1) << 2);
-    const long long d0 = __ldg(lq + phi);
-    const bool nz = valid[s] && d0 != 0ll;
-    const uint32_t m = __ballot_sync(0xffffffffu, nz);
-    if (nz) {
-      SpItemQ e;
-      e.k = k;
-      e.pad = 0u;
-      e.d = (__popc(k & h0.y) & 1) ? -d0 : d0;
-      e.vx = vx[s];
-      e.vy = vy[s];
-      wb[cnt + (uint32_t)__popc(m & lt)] = e;
-    }
-    cnt += (uint32_t)__popc(m);
+__device__ __forceinline__ SpItem<float> sp_item(const SpItem<float>* p) {
+  const uint2 v = __ldg(reinterpret_cast<const uint2*>(p));
+  return {__uint_as_float(v.x), v.y};
+}
+__device__ __forceinline__ SpItem<double> sp_item(const SpItem<double>* p) {
+  const uint4 v = __ldg(reinterpret_cast<const uint4*>(p));
+  return {(long long)(((unsigned long long)v.y << 32) | v.x), v.z, 0u};
+}
+
+// The cases `on` (bit 31 - g) of one head that apply to the lane's amplitude:
+// weight and output offset, sign from sg, product, adds.  A lane walks its own
+// cases, so no slot is spent on a case that does not apply to that lane.  CPLX
+// false: every lane's amplitude has a zero imaginary part (checked by the
+// warp), whose products are zero and are not formed.  acc_s: shared address
+// of the accumulator.
+template <typename R, bool SPLIT, bool CPLX>
+__device__ __forceinline__ void sp_items(const SpItem<R>* __restrict__ it, uint32_t on, uint32_t sg, uint32_t k4,
+                                         typename SpVal<R>::T vx, typename SpVal<R>::T vy, uint32_t acc_s) {
+  while (on) {
+    const int g = __clz(on);
+    on &= ~(0x80000000u >> g);
+    const SpItem<R> e = sp_item(it + g);
+    const typename SpVal<R>::T d = sp_signed(e.w, sg << g);
+    const uint32_t at = acc_s + (k4 ^ e.xo);
+    fx_put<SPLIT, kRe>(at, sp_product(d, vx));
+    if constexpr (CPLX) fx_put<SPLIT, kIm>(at, sp_product(d, vy));
   }
 }
 
-// complex128 term-list group (see sp_terms): the fixed-point weights wq
-// summed exactly, D_q = (sum of all w_q) - 2 (sum of the w_q with odd
-// parity), times the factor 0, 1 or 2, and the complex product in integers.
-template <uint32_t kOct, int A>
-__device__ __forceinline__ void sp_terms_q(const TiledGroup* __restrict__ G, const uint32_t* __restrict__ zs,
-                                           const long long* __restrict__ wq, const uint32_t (&ks)[A],
-                                           const long long (&vx)[A], const long long (&vy)[A],
-                                           const bool (&valid)[A], unsigned long long* acc) {
-  const uint4 g0 = __ldg(reinterpret_cast<const uint4*>(&G->x));     // x, tb, tm, te
-  const uint2 g1 = __ldg(reinterpret_cast<const uint2*>(&G->delta)); // delta, neg
-  uint32_t k[A], fz[A];   // fz: the factor 0, 1 or 2
-  bool on = false;
-#pragma unroll
-  for (int s = 0; s < A; ++s) {
-    k[s] = ks[s] ^ g0.x;
-    fz[s] = 1u;
-    if (g1.x) {
-      const uint32_t p = __popc(k[s] & g1.x) & 1u;
-      fz[s] = (g1.y ? p : p ^ 1u) ? 2u : 0u;
+// The same for the term groups of one head: the weight from the tables (fixed
+// point, summed in integers), s_tab the tile's parts of its groups.
+template <typename R, bool SPLIT>
+__device__ __forceinline__ void sp_tab_items(const SpTab<R>* __restrict__ tab, const typename SpWeight<R>::T* s_tab,
+                                             const SpTables& T, uint32_t on, uint32_t sg, uint32_t kk,
+                                             typename SpVal<R>::T vx, typename SpVal<R>::T vy, bool cplx,
+                                             uint32_t acc_s) {
+  using W = typename SpWeight<R>::T;
+  const uint32_t klow = kk & (kSpTile - 1u);
+  while (on) {
+    const int g = __clz(on);
+    on &= ~(0x80000000u >> g);
+    const SpTab<R>* S = tab + g;
+    W q = s_tab[g] + __ldg(S->fa + (klow & 31u)) + __ldg(S->fb + ((klow >> 5) & 15u)) + __ldg(S->fc + (klow >> 9));
+    const uint4 h = __ldg(reinterpret_cast<const uint4*>(&S->xo));   // xo, x, rb, re
+    for (uint32_t r = h.z; r < h.w; ++r) {
+      const W v = __ldg(reinterpret_cast<const W*>(T.rw) + r);
+      q += (__popc((kk ^ h.y) & __ldg(T.ry + r)) & 1) ? -v : v;
     }
-    on |= valid[s] && fz[s] != 0u;
+    typename SpVal<R>::T d;
+    if constexpr (sizeof(R) == 4) d = (float)q * T.tscale;
+    else d = q;
+    d = sp_signed(d, sg << g);
+    const uint32_t at = acc_s + ((4u * klow) ^ h.x);
+    fx_put<SPLIT, kRe>(at, sp_product(d, vx));
+    if (cplx) fx_put<SPLIT, kIm>(at, sp_product(d, vy));
   }
-  if (!__any_sync(0xffffffffu, on)) return;
-  unsigned long long ar = 0ull, ai = 0ull, odr[A], odi[A];   // modulo 2^64; the results fit
-#pragma unroll
-  for (int s = 0; s < A; ++s) odr[s] = odi[s] = 0ull;
-  for (uint32_t t = g0.y; t < g0.z; ++t) {
-    const uint32_t z = __ldg(zs + t);
-    const unsigned long long w = (unsigned long long)__ldg(wq + t);
-    ar += w;
-#pragma unroll
-    for (int s = 0; s < A; ++s)
-      if (__popc(k[s] & z) & 1) odr[s] += w;
-  }
-  for (uint32_t t = g0.z; t < g0.w; ++t) {
-    const uint32_t z = __ldg(zs + t);
-    const unsigned long long w = (unsigned long long)__ldg(wq + t);
-    ai += w;
-#pragma unroll
-    for (int s = 0; s < A; ++s)
-      if (__popc(k[s] & z) & 1) odi[s] += w;
-  }
-#pragma unroll
-  for (int s = 0; s < A; ++s) {
-    const int sh = fz[s] == 2u ? 1 : 0;
-    const long long a = (long long)((ar - 2ull * odr[s]) << sh), b = (long long)((ai - 2ull * odi[s]) << sh);
-    if (valid[s] && fz[s] != 0u && (a | b) != 0ll)
-      acc_add<kOct>(acc, k[s], q_mul(a, vx[s]) - q_mul(b, vy[s]), q_mul(a, vy[s]) + q_mul(b, vx[s]));
-  }
+}
+
+__device__ __forceinline__ uint4 xor4(const uint4 a, const uint4 b) {
+  return make_uint4(a.x ^ b.x, a.y ^ b.y, a.z ^ b.z, a.w ^ b.w);
+}
+
+// The four parity words of head H at source index klow, with the tile's part
+// b: for the head's 32 cases three loads and 12 XORs in place of 128
+// population counts.
+__device__ __forceinline__ uint4 head_words(const SpHead* __restrict__ H, uint32_t klow, const uint4 b) {
+  return xor4(xor4(__ldg(H->ta + (klow & 31u)), __ldg(H->tb + ((klow >> 5) & 15u))),
+              xor4(__ldg(H->tc + (klow >> 9)), b));
+}
+
+// The factor 0, 1 or 2 of a term-list group at output k (paired groups: 0 or 2).
+__device__ __forceinline__ uint32_t pair_factor(uint32_t k, uint32_t delta, uint32_t neg) {
+  if (!delta) return 1u;
+  const uint32_t p = __popc(k & delta) & 1u;
+  return (neg ? p : p ^ 1u) ? 2u : 0u;
 }
 
 // One term-list group: D(k) = sum_t w_t (-1)^popc(k & z_t), real terms
 // [tb, tm), imaginary [tm, te); a paired group keeps one term of each pair
 // and D = (1 + sigma (-1)^popc(k & delta)) E(k), the factor 0 or 2.  Called
-// by every lane of the warp (the group is warp-uniform).  complex64 (complex128
-// uses sp_terms_q).
-template <typename R, uint32_t kOct, int A, bool SPLIT>
-__device__ __forceinline__ void sp_terms(const TiledGroup* __restrict__ G, const uint32_t* __restrict__ zs,
-                                         const R* __restrict__ ws, const uint32_t (&ks)[A],
-                                         const C_t<R> (&vs)[A], const bool (&valid)[A],
-                                         unsigned long long* acc) {
-  const uint4 g0 = __ldg(reinterpret_cast<const uint4*>(&G->x));     // x, tb, tm, te
-  const uint2 g1 = __ldg(reinterpret_cast<const uint2*>(&G->delta)); // delta, neg
-  uint32_t k[A], fz[A];   // fz: the factor 0, 1 or 2
-  bool on = false;
-#pragma unroll
-  for (int s = 0; s < A; ++s) {
-    k[s] = ks[s] ^ g0.x;
-    fz[s] = 1u;
-    if (g1.x) {
-      const uint32_t p = __popc(k[s] & g1.x) & 1u;
-      fz[s] = (g1.y ? p : p ^ 1u) ? 2u : 0u;
-    }
-    on |= valid[s] && fz[s] != 0u;
+// by every lane of the warp (the group is warp-uniform); kk = k'.
+template <bool SPLIT>
+__device__ __forceinline__ void sp_terms(const SpListGroup& G, const uint32_t* __restrict__ zs,
+                                         const float* __restrict__ ws, uint32_t kk, float vx, float vy, bool valid,
+                                         uint32_t acc_s) {
+  const uint32_t k = kk ^ G.x, fz = pair_factor(k, G.delta, G.neg);
+  if (!__any_sync(0xffffffffu, valid && fz != 0u)) return;
+  float dr = 0.f, di = 0.f;
+  for (uint32_t t = G.tb; t < G.tm; ++t) {
+    const float w = __ldg(ws + t);
+    dr += (__popc(k & __ldg(zs + t)) & 1) ? -w : w;
   }
-  if (!__any_sync(0xffffffffu, on)) return;
-  R dr[A], di[A];
-#pragma unroll
-  for (int s = 0; s < A; ++s) dr[s] = di[s] = R(0);
-  for (uint32_t t = g0.y; t < g0.z; ++t) {
-    const uint32_t z = __ldg(zs + t);
-    const R w = __ldg(ws + t);
-#pragma unroll
-    for (int s = 0; s < A; ++s) dr[s] += (__popc(k[s] & z) & 1) ? -w : w;
+  for (uint32_t t = G.tm; t < G.te; ++t) {
+    const float w = __ldg(ws + t);
+    di += (__popc(k & __ldg(zs + t)) & 1) ? -w : w;
   }
-  for (uint32_t t = g0.z; t < g0.w; ++t) {
-    const uint32_t z = __ldg(zs + t);
-    const R w = __ldg(ws + t);
-#pragma unroll
-    for (int s = 0; s < A; ++s) di[s] += (__popc(k[s] & z) & 1) ? -w : w;
-  }
-#pragma unroll
-  for (int s = 0; s < A; ++s) {
-    const R f = fz[s] == 2u ? R(2) : R(1);
-    const R a = dr[s] * f, b = di[s] * f;
-    if (valid[s] && fz[s] != 0u && (a != R(0) || b != R(0)))
-      acc_add<kOct, SPLIT>(acc, k[s], fx_prod<R>(a * vs[s].x - b * vs[s].y),
-                           fx_prod<R>(a * vs[s].y + b * vs[s].x));
+  const float f = fz == 2u ? 2.f : 1.f;
+  const float a = dr * f, b = di * f;
+  if (valid && fz != 0u && (a != 0.f || b != 0.f)) {
+    const uint32_t at = acc_s + 4u * (k & (kSpTile - 1u));
+    fx_put<SPLIT, kRe>(at, fx_prod(a * vx - b * vy));
+    fx_put<SPLIT, kIm>(at, fx_prod(a * vy + b * vx));
   }
 }
 
-// complex64: a work unit's walk over the piece's LUT groups, then its
-// term-list groups, for the lane's A amplitudes.  Each group's descriptor
-// (x, z0, v0, v1 and v2) is loaded while the group before it is computed.
-template <typename R, uint32_t kOct, int A, bool SPLIT>
-__device__ __forceinline__ void sp_walk(const HLut<R>* __restrict__ ls, int nl, const TiledGroup* __restrict__ gs,
-                                        int nt, const uint32_t* __restrict__ zs, const R* __restrict__ ws,
-                                        const uint32_t (&ks)[A], const C_t<R> (&vs)[A], const bool (&valid)[A],
-                                        unsigned long long* acc) {
-  uint4 h0n = make_uint4(0u, 0u, 0u, 0u);
-  uint32_t v2n = 0u;
-  if (nl > 0) {
-    h0n = __ldg(reinterpret_cast<const uint4*>(&ls[0].x));
-    v2n = __ldg(&ls[0].v2);
+// complex128: the fixed-point weights wq summed exactly,
+// D_q = (sum of all w_q) - 2 (sum of the w_q with odd parity), times the
+// factor 0, 1 or 2, and the complex product in integers.
+template <bool SPLIT>
+__device__ __forceinline__ void sp_terms(const SpListGroup& G, const uint32_t* __restrict__ zs,
+                                         const long long* __restrict__ wq, uint32_t kk, long long vx, long long vy,
+                                         bool valid, uint32_t acc_s) {
+  const uint32_t k = kk ^ G.x, fz = pair_factor(k, G.delta, G.neg);
+  if (!__any_sync(0xffffffffu, valid && fz != 0u)) return;
+  unsigned long long ar = 0ull, ai = 0ull, odr = 0ull, odi = 0ull;   // modulo 2^64; the results fit
+  for (uint32_t t = G.tb; t < G.tm; ++t) {
+    const unsigned long long w = (unsigned long long)__ldg(wq + t);
+    ar += w;
+    if (__popc(k & __ldg(zs + t)) & 1) odr += w;
   }
-  for (int g = 0; g < nl; ++g) {
-    const uint4 h0 = h0n;
-    const uint32_t v2 = v2n;
-    if (g + 1 < nl) {
-      h0n = __ldg(reinterpret_cast<const uint4*>(&ls[g + 1].x));
-      v2n = __ldg(&ls[g + 1].v2);
-    }
-    sp_lut<R, kOct, A, SPLIT>(ls + g, h0, v2, ks, vs, valid, acc);
+  for (uint32_t t = G.tm; t < G.te; ++t) {
+    const unsigned long long w = (unsigned long long)__ldg(wq + t);
+    ai += w;
+    if (__popc(k & __ldg(zs + t)) & 1) odi += w;
   }
-  for (int g = 0; g < nt; ++g) sp_terms<R, kOct, A, SPLIT>(gs + g, zs, ws, ks, vs, valid, acc);
+  const int sh = fz == 2u ? 1 : 0;
+  const long long a = (long long)((ar - 2ull * odr) << sh), b = (long long)((ai - 2ull * odi) << sh);
+  if (valid && fz != 0u && (a | b) != 0ll) {
+    const uint32_t at = acc_s + 4u * (k & (kSpTile - 1u));
+    fx_put<SPLIT, kRe>(at, q_mul(a, vx) - q_mul(b, vy));
+    fx_put<SPLIT, kIm>(at, q_mul(a, vy) + q_mul(b, vx));
+  }
+}
+
+// Terms [m0, m1) of the diagonal group at k (one lane's own amplitude): their
+// sum in 64-bit fixed point times the amplitude as v_q, exact but for one
+// rounding.
+template <bool SPLIT>
+__device__ __forceinline__ void sp_diag(const SpTables& T, uint32_t m0, uint32_t m1, bool imag, uint32_t k, bool on,
+                                        long long vx, long long vy, uint32_t acc_s) {
+  long long d = 0ll;
+#pragma unroll 4
+  for (uint32_t m = m0; m < m1; ++m) {
+    const long long w = __ldg(T.dq + m);
+    d += (__popc(k & __ldg(T.dz + m)) & 1) ? -w : w;
+  }
+  if (!on) return;
+  const uint32_t at = acc_s + 4u * (k & (kSpTile - 1u));
+  const long long pr = imag ? -q_mul(d, vy) : q_mul(d, vx), pi = imag ? q_mul(d, vx) : q_mul(d, vy);
+  if (pr) fx_put_wide<SPLIT, kRe>(at, pr);
+  if (pi) fx_put_wide<SPLIT, kIm>(at, pi);
 }
 
 // 2^e as R, for |e| beyond one float exponent split in two factors.
@@ -560,41 +538,54 @@ __device__ __forceinline__ void pow2_split(int e, R* a, R* b) {
   *b = sizeof(R) == 4 ? (R)ldexpf(1.0f, e2) : (R)ldexp(1.0, e2);
 }
 
+// Shared memory: the accumulator planes, the term groups' tile parts, the
+// first unit of each piece (n_pieces + 1 words) and, when they fit, the heads'
+// tile words.
+constexpr uint32_t kSpMaxSmem = 224u << 10;   // of the 227 KB a block can have
+
+// The part of head q's words that tile t gives.
+__device__ __forceinline__ uint4 tile_words(const SpTables& T, uint32_t q, uint32_t t) {
+  uint4 w = __ldg(T.base + q);
+  for (uint32_t m = t, j = 0; m; m >>= 1, ++j)
+    if (m & 1u) w = xor4(w, __ldg(T.hi + (size_t)j * T.n_sub + q));
+  return w;
+}
+
+// Whether a case of head q can apply in a tile with words b: no parity that
+// the tile decides is one.
+__device__ __forceinline__ bool head_alive(const SpTables& T, uint32_t q, const uint4 b) {
+  const uint4 f = __ldg(T.fix + q);
+  return ~((b.x & f.x) | (b.y & f.y) | (b.z & f.z)) != 0u;
+}
+
 // SPLIT (complex64 only): products added to the accumulator in split form
-// (fx_add_split), converted to 64-bit values before the epilogue.
+// (fx_put), converted to 64-bit values before the epilogue.
 template <typename R, bool SPLIT>
-__global__ void __launch_bounds__(sp_threads<R>(), 1) k_apply_h_sparse(const SparseArgs<R> a) {
+__global__ void __launch_bounds__(kSpThreads, 1) k_apply_h_sparse(const SparseArgs<R> a) {
   static_assert(!SPLIT || sizeof(R) == 4, "the split accumulator takes 32-bit products");
-  constexpr int LB = TiledBits<R>::LB;
-  constexpr int NT = sp_threads<R>();
-  constexpr int A = sp_amps<R>();             // amplitudes per lane per work unit
-  constexpr uint32_t kChunk = 32u * A;        // amplitudes per work unit
-  constexpr uint32_t kOct = 1u << (LB - 3);   // octets per tile
+  constexpr int NT = kSpThreads;
   if (*a.alen > a.max_amps) return;           // the staged kernel takes this state
-  // dynamic shared memory: the tile's fixed-point accumulator, 16 components
-  // x kOct octets of 8 bytes
+  using W = typename SpWeight<R>::T;
   extern __shared__ __align__(16) uint8_t sp_raw[];
-  unsigned long long* acc = reinterpret_cast<unsigned long long*>(sp_raw);
+  uint8_t* acc = sp_raw;
+  const uint32_t acc_s = smem_u32(acc);
+  const uint32_t P = (uint32_t)a.sp.n_pieces;
+  uint4* s_base = reinterpret_cast<uint4*>(sp_raw + kAccBytes);
+  W* s_tab = reinterpret_cast<W*>(s_base + (a.base_smem ? a.sp.n_sub : 0u));
+  uint32_t* s_pre = reinterpret_cast<uint32_t*>(s_tab + a.sp.n_tab);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  // complex128: the warp's item buffer after the accumulator
-  SpItemQ* wb = reinterpret_cast<SpItemQ*>(sp_raw + kOct * 16u * sizeof(unsigned long long)) +
-                (sizeof(R) == 8 ? warp * kSpCapQ : 0u);
-  const uint32_t lt = (1u << lane) - 1u;
-  uint32_t cnt = 0;   // items in wb (warp-uniform)
-  // complex128: the fixed-point copy of a blob byte is at the same offset
-  // from a.wfix as the byte from a.blob
-  const ptrdiff_t wdelta = a.wfix - a.blob;
   __shared__ uint32_t s_tile, s_unext;
-  __shared__ uint32_t s_pre[kSpMaxPieces + 1];   // first unit of each piece; s_pre[P] = units
   __shared__ uint32_t s_wsum[32];
   __shared__ double s_red[2][NT / 32];
   __shared__ bool s_last;
-  const uint32_t ntiles = 1u << (a.n - LB);
-  const uint32_t P = (uint32_t)a.n_pieces;
-  for (uint32_t j = threadIdx.x; j < kOct * 16u; j += NT) acc[j] = 0ull;
-  // fixed-point scale 2^F: every sum below 2^62 (hbound x 2 max|component|
-  // x 2^F <= 2^62) and, for complex64, every off-diagonal product below 2^30
-  // (dmax x 2 max|component| x 2^F <= 2^30)
+  const uint32_t ntiles = a.n > kSpLB ? 1u << (a.n - kSpLB) : 1u;
+  const uint32_t n_oct = a.n > kSpLB ? kSpTile / 8u : 1u << (a.n - 3);   // octets of a tile
+  const bool base_smem = a.base_smem;
+  for (uint32_t j = threadIdx.x; j < kAccBytes / 16u; j += NT)
+    reinterpret_cast<uint4*>(acc)[j] = make_uint4(0u, 0u, 0u, 0u);
+  // fixed-point scale 2^F: every sum below 2^62 (complex64: 2^46), hbound x
+  // 2 max|component| x 2^F, and, for complex64, every off-diagonal product
+  // below 2^30 (dmax x 2 max|component| x 2^F <= 2^30)
   int F = 0;
   {
     const double m = __longlong_as_double((long long)*a.amax);
@@ -602,7 +593,7 @@ __global__ void __launch_bounds__(sp_threads<R>(), 1) k_apply_h_sparse(const Spa
     if (bnd > 0.0) {
       int e;
       frexp(bnd, &e);   // bnd < 2^e
-      F = 62 - e;
+      F = (sizeof(R) == 4 ? 46 : 62) - e;
       if (sizeof(R) == 4 && bnd1 > 0.0) {
         frexp(bnd1, &e);
         F = min(F, 30 - e);
@@ -613,7 +604,6 @@ __global__ void __launch_bounds__(sp_threads<R>(), 1) k_apply_h_sparse(const Spa
   pow2_split<R>(F, &up_a, &up_b);
   pow2_split<R>(-F, &dn_a, &dn_b);
   const double dn = ldexp(1.0, -F);
-  const R idr = (R)a.identity;
   const uint32_t K = a.parts;   // blocks per output tile
   for (;;) {
     if (threadIdx.x == 0) {
@@ -626,18 +616,40 @@ __global__ void __launch_bounds__(sp_threads<R>(), 1) k_apply_h_sparse(const Spa
     // the claim is part `part` of output tile t: the part takes the tile's
     // unit batches part, part + K, part + 2K, ...
     const uint32_t t = claim / K, part = claim - t * K;
-    // Work units are (piece p, chunk c): the nonzero amplitudes kChunk c ..
-    // kChunk (c + 1) - 1 of p's source tile u = t ^ (x >> LB) against p's
-    // groups, numbered piece by piece (s_pre: a block scan of the chunk counts).
+    // Work units are (piece p, span of chunks): 32 span consecutive nonzero
+    // amplitudes of p's source tile u = t ^ (x >> LB) against p's groups,
+    // numbered piece by piece (s_pre: a block scan of the unit counts).
+    // A piece of few sub-blocks takes several chunks per unit, so that
+    // finding and starting a unit stays small beside its work; small states
+    // (K > 1), which have few units, take one.
     {
-      const uint32_t per = (P + NT - 1) / NT, p0 = threadIdx.x * per, p1 = min(P, p0 + per);
+      // the tile's part of each head's parities and of each term group's weight
+      if (base_smem)
+        for (uint32_t q = threadIdx.x; q < a.sp.n_sub; q += NT) s_base[q] = tile_words(a.sp, q, t);
+      for (uint32_t q = threadIdx.x; q < a.sp.n_tab; q += NT) {
+        const SpTabTile<R> tt = reinterpret_cast<const SpTabTile<R>*>(a.sp.tile)[q];
+        W f = tt.f0;
+        for (uint32_t h = tt.hb; h < tt.he; ++h) {
+          const W v = __ldg(reinterpret_cast<const W*>(a.sp.hw) + h);
+          f += (__popc(t & __ldg(a.sp.hy + h)) & 1) ? -v : v;
+        }
+        s_tab[q] = f;
+      }
+      __syncthreads();
+      const uint32_t per = (P + NT - 1) / NT, p0 = min(P, threadIdx.x * per), p1 = min(P, p0 + per);
       uint32_t mine = 0;
       for (uint32_t p = p0; p < p1; ++p) {
-        const TiledPiece pc = a.piece[a.porder[p]];
-        const uint32_t u = t ^ pc.xhi;
-        const uint32_t nch = pc.bytes ? (a.toff[u + 1] - a.toff[u] + kChunk - 1u) / kChunk : 0u;
-        s_pre[p] = nch;
-        mine += nch;
+        const SpPiece pc = a.sp.piece[p];
+        const uint32_t u = t ^ pc.xhi, cs = 32u * (K > 1u ? 1u : pc.span);
+        uint32_t nu = (a.toff[u + 1] - a.toff[u] + cs - 1u) / cs;
+        if (nu && pc.kind < 2) {   // a piece none of whose cases can apply in this tile has no units
+          bool alive = false;
+          for (uint32_t q = pc.sub0; q < pc.sub0 + pc.nsub && !alive; ++q)
+            alive = head_alive(a.sp, q, base_smem ? s_base[q] : tile_words(a.sp, q, t));
+          if (!alive) nu = 0u;
+        }
+        s_pre[p] = nu;
+        mine += nu;
       }
       uint32_t incl = mine;
       for (int o = 1; o < 32; o <<= 1) {
@@ -647,41 +659,41 @@ __global__ void __launch_bounds__(sp_threads<R>(), 1) k_apply_h_sparse(const Spa
       if (lane == 31) s_wsum[warp] = incl;
       __syncthreads();
       if (warp == 0) {
-        uint32_t ws = lane < NT / 32 ? s_wsum[lane] : 0u, wi = ws;
+        uint32_t ws = s_wsum[lane], wi = ws;
         for (int o = 1; o < 32; o <<= 1) {
           const uint32_t q = __shfl_up_sync(0xffffffffu, wi, o);
           if (lane >= o) wi += q;
         }
-        if (lane < NT / 32) s_wsum[lane] = wi - ws;   // exclusive
-        if (lane == NT / 32 - 1) s_pre[P] = wi;
+        s_wsum[lane] = wi - ws;   // exclusive
+        if (lane == 31) s_pre[P] = wi;
       }
       __syncthreads();
       uint32_t run = s_wsum[warp] + incl - mine;
       for (uint32_t p = p0; p < p1; ++p) {
-        const uint32_t nch = s_pre[p];
+        const uint32_t nu = s_pre[p];
         s_pre[p] = run;
-        run += nch;
+        run += nu;
       }
     }
     __syncthreads();
     const uint32_t n_units = s_pre[P];
-    // kUnitBatch consecutive units per claim (mostly chunks of one piece,
-    // whose descriptors then stay in L1); one per claim when the tile has
-    // fewer than kUnitBatch units per warp of its K blocks, so that the few
-    // units of a small state do not queue behind each other on one warp
-    const uint32_t batch = n_units < kUnitBatch * (uint32_t)(NT / 32) * K ? 1u : kUnitBatch;
+    // kUnitBatch consecutive units per claim (mostly of one piece, whose
+    // tables then stay in L1), single ones towards the end of a tile and for
+    // the few units of a small state (K > 1): a warp that starts a batch when
+    // the others find none left keeps the whole block waiting
+    uint32_t j0 = 0, p = 0;
     for (;;) {
-      uint32_t j0 = 0;
-      if (lane == 0) j0 = (atomicAdd(&s_unext, 1u) * K + part) * batch;
+      // units left when this warp claimed last decide how many it takes now
+      const uint32_t batch = K == 1u && n_units - j0 > 8u * kUnitBatch * (uint32_t)(NT / 32) ? kUnitBatch : 1u;
+      if (lane == 0) j0 = atomicAdd(&s_unext, batch) * K + part;
       j0 = __shfl_sync(0xffffffffu, j0, 0);
       if (j0 >= n_units) break;
       const uint32_t j1 = min(n_units, j0 + batch);
       // p = the last piece with s_pre[p] <= j0 (pieces without units share
-      // their successor's start and are passed over), then advanced along
-      // the batch
-      uint32_t p;
-      {
-        uint32_t lo = 0, hi = P - 1;
+      // their successor's start and are passed over), from the last claim's
+      // piece on, then advanced along the batch
+      if (s_pre[p + 1] <= j0) {
+        uint32_t lo = p + 1, hi = P - 1;
         while (lo < hi) {
           const uint32_t mid = (lo + hi + 1) >> 1;
           if (s_pre[mid] <= j0) lo = mid;
@@ -691,83 +703,59 @@ __global__ void __launch_bounds__(sp_threads<R>(), 1) k_apply_h_sparse(const Spa
       }
       for (uint32_t j = j0; j < j1; ++j) {
         while (p + 1 < P && s_pre[p + 1] <= j) ++p;
-        const uint32_t c = j - s_pre[p];
-        const uint32_t pid = a.porder[p];
-        const TiledPiece pc = a.piece[pid];
-        const uint32_t u = t ^ pc.xhi;
-        const uint32_t a0 = a.toff[u], a1 = a.toff[u + 1];
-        const uint8_t* blob = a.blob + pc.off;
-        const uint4 hd = __ldg(reinterpret_cast<const uint4*>(blob));   // n_runs, n_lut, z_off, w_off
-        const HLut<R>* ls = reinterpret_cast<const HLut<R>*>(blob + sizeof(TiledHead));
-        const TiledGroup* gs = reinterpret_cast<const TiledGroup*>(blob + sizeof(TiledHead) + hd.y * sizeof(HLut<R>));
-        const uint32_t* zs = reinterpret_cast<const uint32_t*>(blob + hd.z);
-        const R* ws = reinterpret_cast<const R*>(blob + hd.w);
-        uint32_t ks[A];
-        C_t<R> vs[A];
-        long long vqx[A], vqy[A];   // complex128: the amplitudes as v_q (see q_mul)
-        bool valid[A];
-#pragma unroll
-        for (int s = 0; s < A; ++s) {
-          const uint32_t li = a0 + kChunk * c + 32u * s + (uint32_t)lane;
-          valid[s] = li < a1;
-          ks[s] = a.aidx[valid[s] ? li : a0];
-          const C_t<R> v = a.aval[valid[s] ? li : a0];
-          vs[s] = cmake<R>(v.x * up_a * up_b, v.y * up_a * up_b);
-          if constexpr (sizeof(R) == 8) {
-            vqx[s] = __double2ll_rn((double)vs[s].x * a.wscale);
-            vqy[s] = __double2ll_rn((double)vs[s].y * a.wscale);
+        const SpPiece pc = a.sp.piece[p];
+        const uint32_t u = t ^ pc.xhi, cs = 32u * (K > 1u ? 1u : pc.span);
+        const uint32_t l0 = a.toff[u] + (j - s_pre[p]) * cs, a1 = min(a.toff[u + 1], l0 + cs);
+        for (uint32_t l = l0; l < a1; l += 32u) {
+          const uint32_t li = l + (uint32_t)lane;
+          const bool valid = li < a1;
+          const uint32_t kk = a.aidx[valid ? li : l];
+          const C_t<R> v = a.aval[valid ? li : l];
+          typename SpVal<R>::T vx, vy;
+          if constexpr (sizeof(R) == 4) {
+            vx = v.x * up_a * up_b;
+            vy = v.y * up_a * up_b;
+          } else {
+            vx = __double2ll_rn(v.x * up_a * up_b * a.sp.wscale);
+            vy = __double2ll_rn(v.y * up_a * up_b * a.sp.wscale);
           }
-        }
-        const int nl = (int)hd.y;
-        // the term-list groups fill the blob from the LUT groups to z_off
-        const int nt = (int)((hd.z - sizeof(TiledHead) - nl * sizeof(HLut<R>)) / sizeof(TiledGroup));
-        if constexpr (sizeof(R) == 8) {
-          // each group's descriptor (x, z0, v0, v1 and v2) is loaded while
-          // the group before it is computed
-          uint4 h0n = make_uint4(0u, 0u, 0u, 0u);
-          uint32_t v2n = 0u;
-          if (nl > 0) {
-            h0n = __ldg(reinterpret_cast<const uint4*>(&ls[0].x));
-            v2n = __ldg(&ls[0].v2);
-          }
-          for (int g = 0; g < nl; ++g) {
-            const uint4 h0 = h0n;
-            const uint32_t v2 = v2n;
-            if (g + 1 < nl) {
-              h0n = __ldg(reinterpret_cast<const uint4*>(&ls[g + 1].x));
-              v2n = __ldg(&ls[g + 1].v2);
+          const bool cplx = __any_sync(0xffffffffu, valid && !rzero<R>(v.y));
+          const uint32_t on = valid ? ~0u : 0u, klow = kk & (kSpTile - 1u);
+          if (pc.kind < 2) {
+            for (uint32_t q = pc.sub0; q < pc.sub0 + pc.nsub; ++q) {
+              const uint4 w = head_words(a.sp.head + q, klow, base_smem ? s_base[q] : tile_words(a.sp, q, t));
+              const uint32_t cases = ~(w.x | w.y | w.z) & on;
+              if (pc.kind == 0) {
+                const SpItem<R>* it = reinterpret_cast<const SpItem<R>*>(a.sp.item) + (size_t)kSpCases * q;
+                if (cplx) sp_items<R, SPLIT, true>(it, cases, w.w, 4u * klow, vx, vy, acc_s);
+                else sp_items<R, SPLIT, false>(it, cases, w.w, 4u * klow, vx, vy, acc_s);
+              } else {
+                const uint32_t slot = pc.tab0 + kSpCases * (q - pc.sub0);
+                sp_tab_items<R, SPLIT>(reinterpret_cast<const SpTab<R>*>(a.sp.tab) + slot, s_tab + slot, a.sp, cases,
+                                       w.w, kk, vx, vy, cplx, acc_s);
+              }
+              __syncwarp();   // the lanes' walks differ in length: the next head starts together
             }
-            const long long* lq = reinterpret_cast<const long long*>(
-                reinterpret_cast<const uint8_t*>(ls[g].lut16) + wdelta);
-            sp_lut_q<kOct, A>(lq, h0, v2, ks, vqx, vqy, valid, wb, cnt, lt);
-            while (cnt >= 32u) {
-              cnt -= 32u;
-              sp_flush_q<kOct>(wb, cnt + (uint32_t)lane, true, acc);
-            }
+          } else if (pc.kind != 2) {
+            // the own tile's amplitudes (pc.xhi = 0) times diagonal terms
+            const long long wx = __double2ll_rn((double)(v.x * up_a * up_b) * a.sp.dscale);
+            const long long wy = __double2ll_rn((double)(v.y * up_a * up_b) * a.sp.dscale);
+            sp_diag<SPLIT>(a.sp, pc.sub0, pc.sub0 + pc.nsub, pc.kind == 4, kk, valid, wx, wy, acc_s);
+          } else {
+            for (uint32_t g = pc.sub0; g < pc.sub0 + pc.nsub; ++g)
+              sp_terms<SPLIT>(a.sp.list[g], a.sp.lz, reinterpret_cast<const typename SpVal<R>::T*>(a.sp.lw), kk, vx,
+                              vy, valid, acc_s);
           }
-          const long long* wq = reinterpret_cast<const long long*>(reinterpret_cast<const uint8_t*>(ws) + wdelta);
-          for (int g = 0; g < nt; ++g) sp_terms_q<kOct, A>(gs + g, zs, wq, ks, vqx, vqy, valid, acc);
-        } else if (A > 1 && a0 + kChunk * c + 32u >= a1) {
-          // the unit's amplitudes fill the first lane slot at most (the last
-          // chunk of a source tile): the groups are walked for that slot
-          // alone instead of issuing the empty slots with every lane idle
-          const uint32_t ks1[1] = {ks[0]};
-          const C_t<R> vs1[1] = {vs[0]};
-          const bool valid1[1] = {valid[0]};
-          sp_walk<R, kOct, 1, SPLIT>(ls, nl, gs, nt, zs, ws, ks1, vs1, valid1, acc);
-        } else {
-          sp_walk<R, kOct, A, SPLIT>(ls, nl, gs, nt, zs, ws, ks, vs, valid, acc);
         }
       }
     }
-    if (cnt) sp_flush_q<kOct>(wb, (uint32_t)lane, (uint32_t)lane < cnt, acc);   // the rest, fewer than 32
-    cnt = 0;
     __syncthreads();
     if constexpr (SPLIT) {
-      // every product is in: the split words become 64-bit values
-      for (uint32_t j = threadIdx.x; j < kOct * 16u; j += NT) {
-        const unsigned long long v = acc[j];
-        if (v) acc[j] = split_to_wide(v);
+      // every product is in: the split halves become 64-bit values
+      for (uint32_t j = threadIdx.x; j < 2u * kSpTile; j += NT) {
+        const uint32_t at = 4u * (j & (kSpTile - 1u)) + (j & kSpTile ? kIm : kRe);
+        const long long v = acc_get(acc, at);   // high half | low half
+        if (v) acc_set(acc, at, (v >> 32) * 65536ll + (v & 0xffffffffll));
       }
       __syncthreads();
     }
@@ -776,59 +764,44 @@ __global__ void __launch_bounds__(sp_threads<R>(), 1) k_apply_h_sparse(const Spa
       // to the tile's global accumulator (64-bit integer atomics: the same
       // sum in any order), and the last to finish takes the total, clears
       // the global copy for the next call and runs the epilogue
-      unsigned long long* g = a.gacc + (size_t)t * (kOct * 16u);
-      for (uint32_t j = threadIdx.x; j < kOct * 16u; j += NT) {
-        const unsigned long long v = acc[j];
-        if (v) atomicAdd(g + j, v);
+      unsigned long long* g = a.gacc + (size_t)t * (2u * kSpTile);
+      for (uint32_t j = threadIdx.x; j < 2u * kSpTile; j += NT) {
+        const long long v = acc_get(acc, 4u * (j & (kSpTile - 1u)) + (j & kSpTile ? kIm : kRe));
+        if (v) atomicAdd(g + j, (unsigned long long)v);
       }
       __threadfence();
       __syncthreads();
       if (threadIdx.x == 0) s_last = atomicAdd(a.tdone + t, 1u) == K - 1u;
       __syncthreads();
       if (!s_last) {
-        for (uint32_t j = threadIdx.x; j < kOct * 16u; j += NT) acc[j] = 0ull;
+        for (uint32_t j = threadIdx.x; j < kAccBytes / 16u; j += NT)
+          reinterpret_cast<uint4*>(acc)[j] = make_uint4(0u, 0u, 0u, 0u);
         __syncthreads();
         continue;
       }
       __threadfence();
-      for (uint32_t j = threadIdx.x; j < kOct * 16u; j += NT) {
-        acc[j] = __ldcg(g + j);
+      for (uint32_t j = threadIdx.x; j < 2u * kSpTile; j += NT) {
+        acc_set(acc, 4u * (j & (kSpTile - 1u)) + (j & kSpTile ? kIm : kRe), (long long)__ldcg(g + j));
         __stcg(g + j, 0ull);
       }
       if (threadIdx.x == 0) a.tdone[t] = 0u;
       __syncthreads();
     }
-    // epilogue, first the nonzero amplitudes of the own tile (one lane
-    // each): the diagonal group and the identity, which act on psi(k) alone,
-    // and the energy partials (zero amplitudes add to neither); each k is
-    // one lane's, so its accumulator entry is updated without atomics
+    // epilogue, first the energy partials over the nonzero amplitudes of the
+    // own tile (zero amplitudes add nothing): one full warp of amplitudes at a
+    // time, since the FP64 pipe is narrow here
     {
-      double2 w = make_double2(0.0, 0.0);   // this thread's |psi|^2 and <psi|H - identity|psi> partials
-      const uint32_t e0 = a.toff[t], e1 = a.toff[t + 1];
+      double2 w = make_double2(0.0, 0.0);   // this thread's |psi|^2 and Re<psi|H psi> partials
+      const uint32_t e0 = a.toff[t], e1 = a.partials ? a.toff[t + 1] : e0;
       for (uint32_t e = e0 + threadIdx.x; e < e1; e += NT) {
-        const uint32_t k = a.aidx[e];
         const C_t<R> q = a.aval[e];
-        R dr = R(0), dc = R(0), di = R(0);
-        for (int m = 0; m < a.nd_mid; ++m) {
-          const R y = ((__popc(k & a.dz[m]) & 1) ? -a.dw[m] : a.dw[m]) - dc;
-          if (sizeof(R) == 4) {   // compensated in FP32
-            const R s2 = dr + y;
-            dc = (s2 - dr) - y;
-            dr = s2;
-          } else {
-            dr += y;
-          }
+        const uint32_t at = 4u * (a.aidx[e] & (kSpTile - 1u));
+        w.x += (double)q.x * q.x;
+        w.y += (double)q.x * ((double)acc_get(acc, at + kRe) * dn);
+        if (!rzero<R>(q.y)) {
+          w.x += (double)q.y * q.y;
+          w.y += (double)q.y * ((double)acc_get(acc, at + kIm) * dn);
         }
-        for (int m = a.nd_mid; m < a.nd; ++m) di += (__popc(k & a.dz[m]) & 1) ? -a.dw[m] : a.dw[m];
-        unsigned long long* e2 = acc + acc_at<kOct>(k);
-        const double ox = (double)(long long)e2[0] * dn, oy = (double)(long long)e2[kOct] * dn;
-        const double pp = (double)q.x * q.x + (double)q.y * q.y;
-        w.x += pp;
-        w.y += (double)q.x * ox + (double)q.y * oy + ((double)dr - (double)dc) * pp;
-        const R d0 = dr - dc + idr;
-        const C_t<R> qs = cmake<R>(q.x * up_a * up_b, q.y * up_a * up_b);
-        e2[0] = (unsigned long long)((long long)e2[0] + fx_wide<R>(d0 * qs.x - di * qs.y));
-        e2[kOct] = (unsigned long long)((long long)e2[kOct] + fx_wide<R>(d0 * qs.y + di * qs.x));
       }
       // the tile's energy partials, summed in a fixed order (warps that
       // hold no amplitude of the tile skip the FP64 shuffles)
@@ -848,16 +821,27 @@ __global__ void __launch_bounds__(sp_threads<R>(), 1) k_apply_h_sparse(const Spa
       a.partials[2u * t + threadIdx.x] = sum;
     }
     // then the whole tile out (zeros included) and the accumulator cleared
-    for (uint32_t o = threadIdx.x; o < kOct; o += NT) {
-      const uint32_t k0 = ((t << (LB - 3)) | o) << 3;
+    for (uint32_t o = threadIdx.x; o < n_oct; o += NT) {
+      const uint32_t k0 = t * kSpTile + 8u * o;
       C_t<R> res[kAmpsH];
 #pragma unroll
-      for (int i = 0; i < kAmpsH; ++i) {
-        unsigned long long* e = acc + acc_at<kOct>(k0 | (uint32_t)i);
-        const R re = fx_val<R>(e[0]), im = fx_val<R>(e[kOct]);
-        res[i] = cmake<R>(re * dn_a * dn_b, im * dn_a * dn_b);
-        e[0] = 0ull;
-        e[kOct] = 0ull;
+      for (int h = 0; h < kAmpsH; h += 4) {   // four amplitudes of each plane at a time
+        const uint32_t at = 4u * (8u * o + h);
+        uint4 pl[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          uint4* e = reinterpret_cast<uint4*>(acc + at + q * kPlane);
+          pl[q] = *e;
+          *e = make_uint4(0u, 0u, 0u, 0u);
+        }
+        const uint32_t rl[4] = {pl[0].x, pl[0].y, pl[0].z, pl[0].w}, rh[4] = {pl[1].x, pl[1].y, pl[1].z, pl[1].w};
+        const uint32_t il[4] = {pl[2].x, pl[2].y, pl[2].z, pl[2].w}, ih[4] = {pl[3].x, pl[3].y, pl[3].z, pl[3].w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const R re = fx_val<R>((long long)(((unsigned long long)rh[i] << 32) | rl[i]));
+          const R im = fx_val<R>((long long)(((unsigned long long)ih[i] << 32) | il[i]));
+          res[h + i] = cmake<R>(re * dn_a * dn_b, im * dn_a * dn_b);
+        }
       }
       C_t<R>* dst = a.out + k0;
       if (sizeof(R) == 4) {
@@ -902,36 +886,29 @@ __global__ void __launch_bounds__(sp_threads<R>(), 1) k_apply_h_sparse(const Spa
       eh += s_red[1][q];
     }
     a.scal[1] = n2;
-    a.scal[2] = eh;
-    a.scal[0] = a.identity + eh / n2;
+    a.scal[2] = eh - a.identity * n2;
+    a.scal[0] = eh / n2;
     *a.counter = 0u;
   }
-}
-
-template <typename R>
-constexpr uint32_t sparse_smem() {
-  return (1u << (TiledBits<R>::LB - 3)) * 16u * (uint32_t)sizeof(unsigned long long) +
-         (sizeof(R) == 8 ? (uint32_t)(sp_threads<R>() / 32) * kSpCapQ * (uint32_t)sizeof(SpItemQ) : 0u);
 }
 
 }  // namespace
 
 template <typename R>
 int sparse_apply_h(SparseArgs<R> a, const LiveOctets& lv, int sm_count, cudaStream_t st) {
-  constexpr int LB = TiledBits<R>::LB;
-  if (a.n < LB || !lv.toff || !lv.aidx || !lv.aval || !lv.alen || !lv.acounts || !lv.amax || a.max_amps > lv.acap)
-    return fail(GOCP_EINVAL, "scatter H psi needs the amplitude list");
-  if (sizeof(R) == 8 && !a.wfix) return fail(GOCP_EINVAL, "scatter H psi (complex128) needs the fixed-point weights");
+  if (!lv.toff || !lv.aidx || !lv.aval || !lv.alen || !lv.acounts || !lv.amax || a.max_amps > lv.acap || a.sp.n_pieces <= 0)
+    return fail(GOCP_EINVAL, "scatter H psi needs the amplitude list and its tables");
   a.amax = lv.amax;
   a.aidx = lv.aidx;
   a.aval = reinterpret_cast<const C_t<R>*>(lv.aval);
   a.alen = lv.alen;
   a.toff = lv.toff;
   // complex64 adds its products in split form when every accumulator word
-  // takes fewer than 65536 of them (one per off-diagonal group); the two
+  // takes fewer than 65536 of them (at most one per off-diagonal group and
+  // diagonal piece); the two
   // forms give the same integers, so H psi does not depend on the choice
   // (GOCP_SCATTER_SPLIT=0 selects the carry form)
-  bool split = sizeof(R) == 4 && a.n_offdiag < 65536u;
+  bool split = sizeof(R) == 4 && a.n_offdiag + (uint32_t)a.sp.n_pieces < 65536u;
   if (const char* ev = std::getenv("GOCP_SCATTER_SPLIT"))
     if (ev[0] == '0') split = false;
   auto kern = split ? k_apply_h_sparse<R, sizeof(R) == 4> : k_apply_h_sparse<R, false>;
@@ -945,27 +922,22 @@ int sparse_apply_h(SparseArgs<R> a, const LiveOctets& lv, int sm_count, cudaStre
     if (device >= (int)done.size()) done.resize(device + 1, false);
     if (!done[device]) {
       e = cudaFuncSetAttribute(k_apply_h_sparse<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)sparse_smem<R>());
+                               (int)kSpMaxSmem);
       if (e == cudaSuccess && sizeof(R) == 4)
         e = cudaFuncSetAttribute(k_apply_h_sparse<R, sizeof(R) == 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sparse_smem<R>());
+                                 (int)kSpMaxSmem);
       if (e != cudaSuccess) return cuda_status(e, "cudaFuncSetAttribute(k_apply_h_sparse)");
       done[device] = true;
     }
   }
   int rc = amp_list(sizeof(R) == 4 ? GOCP_C64 : GOCP_C128, a.psi, a.mask, a.n, lv, st);
   if (rc) return rc;
-  const uint32_t ntiles = 1u << (a.n - LB);
-  k_tile_offsets<<<(ntiles + 256u) / 256u, 256, 0, st>>>(lv.aidx, lv.alen, lv.acap, ntiles, LB, lv.toff);
+  const uint32_t ntiles = a.n > kSpLB ? 1u << (a.n - kSpLB) : 1u;
+  k_tile_offsets<<<(ntiles + 256u) / 256u, 256, 0, st>>>(lv.aidx, lv.alen, lv.acap, ntiles, kSpLB, lv.toff);
   // tiles for fewer than half the SMs: K blocks share each tile (K a power
   // of two up to 64, or GOCP_SCATTER_PARTS, so that ntiles K reaches the SM
   // count), combining their fixed-point accumulators in global memory; the
-  // sums are integer, so H psi and E do not depend on K.  Measured per H psi
-  // call on prepared ADAPT states (complex64 / complex128): 14 qubits
-  // 0.19 / 0.23 -> 0.14 / 0.17 ms, 16 qubits 0.27 / 0.33 -> 0.20 / 0.20 ms,
-  // 18 qubits 0.34 / 0.42 -> 0.22 / 0.30 ms; with 128 tiles on 152 SMs
-  // (20 qubits complex64) splitting was slower, and two waves of parts
-  // slower than one.
+  // sums are integer, so H psi and E do not depend on K.
   const uint32_t sms = (uint32_t)std::max(sm_count, 1);
   uint32_t kmax = 64u;
   if (const char* e = std::getenv("GOCP_SCATTER_PARTS")) {
@@ -979,7 +951,12 @@ int sparse_apply_h(SparseArgs<R> a, const LiveOctets& lv, int sm_count, cudaStre
   a.gacc = lv.gacc;
   a.tdone = lv.tdone;
   const int grid = (int)std::min<uint64_t>((uint64_t)ntiles * K, (uint64_t)sms);
-  kern<<<grid, sp_threads<R>(), sparse_smem<R>(), st>>>(a);
+  static_assert(kAccBytes + 8u * kSpMaxTab + 4u * (kSpMaxPieces + 1u) <= kSpMaxSmem, "the tables fit beside the planes");
+  uint32_t smem = kAccBytes + (uint32_t)sizeof(typename SpWeight<R>::T) * a.sp.n_tab +
+                  4u * ((uint32_t)a.sp.n_pieces + 1u);
+  a.base_smem = (uint64_t)smem + 16ull * a.sp.n_sub <= kSpMaxSmem;
+  if (a.base_smem) smem += 16u * a.sp.n_sub;
+  kern<<<grid, kSpThreads, smem, st>>>(a);
   count_launches(2);
   return cuda_status(cudaGetLastError(), "k_apply_h_sparse");
 }

@@ -678,15 +678,12 @@ int launch_tiled(const DevTables& t, const LiveOctets& lv, int sm_count, const v
   // states with few nonzero amplitudes: the scatter kernel (the staged one
   // then returns at once); the choice is made on the device from the count
   const double frac = sparse_frac();
-  const bool scatter = frac > 0.0 && lv.aidx && lv.toff && t.n_pieces <= kSpMaxPieces;
+  const bool scatter = frac > 0.0 && lv.aidx && lv.toff && t.sp.n_pieces > 0;
   const uint32_t max_amps =
       (uint32_t)std::min<double>((double)lv.acap, std::floor(frac * (double)(1ull << t.n)));
   if (scatter) {
     SparseArgs<R> s;
-    s.blob = t.tblob;
-    s.piece = t.tpiece;
-    s.porder = t.tporder;
-    s.n_pieces = t.n_pieces;
+    s.sp = t.sp;
     s.n = t.n;
     s.psi = reinterpret_cast<const C_t<R>*>(psi);
     s.out = reinterpret_cast<C_t<R>*>(hpsi);
@@ -695,12 +692,6 @@ int launch_tiled(const DevTables& t, const LiveOctets& lv, int sm_count, const v
     s.n_offdiag = (uint32_t)(t.G + t.GL);
     s.hbound = t.hbound;
     s.dmax = t.dmax;
-    s.wfix = t.twfix;
-    s.wscale = t.twscale;
-    s.dz = t.dz;
-    s.dw = reinterpret_cast<const R*>(t.dw);
-    s.nd = t.nd;
-    s.nd_mid = t.nd_mid;
     s.identity = identity;
     s.partials = partials;
     s.counter = counter;

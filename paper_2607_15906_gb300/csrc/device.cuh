@@ -198,6 +198,97 @@ struct __align__(16) TiledPiece {
   uint32_t xhi, off, bytes, pad;
 };
 
+// Scatter H psi (apply_sparse.cu).  Output tiles of 2^kSpLB amplitudes.  An
+// off-diagonal LUT group is split into *cases*: a case holds where up to three
+// parities of the output index k are zero (an affine subspace of the group's
+// codes on which the weight has one magnitude), with the weight
+// w (-1)^sigma(k), sigma a fourth parity.  A two-electron group of a molecular
+// H gives one case (two alpha and two beta orbitals) or three (four orbitals
+// of one spin).  The cases of equal x >> kSpLB are cut into heads of 32; for
+// source index k' the head's four words (bit 31 - g: parity of case g) are
+// linear in the bits of k', so they are the XOR of the tile's part
+// (SpTables::base, which also folds in k = k' ^ x, and hi per bit of the tile
+// number) and of table entries for bits 0..4, 5..8 and 9..12 of k'.  The cases
+// that apply are then ~(p0 | p1 | p2).  Unused cases have p0 = 1.
+constexpr int kSpLB = 13;
+constexpr uint32_t kSpTile = 1u << kSpLB;
+constexpr int kSpCases = 32;
+template <typename R> struct SpWeight;
+template <> struct SpWeight<float> { using T = int32_t; };      // round(w 2^Ft)
+template <> struct SpWeight<double> { using T = long long; };   // round(w 2^Fd)
+struct __align__(16) SpHead {
+  uint4 ta[32], tb[16], tc[16];   // x, y, z: the parities p0, p1, p2; w: the sign
+};
+// A case's weight and offset 4 (x mod 2^kSpLB).  complex128 weights are
+// round(w 2^Fd), Fd = 62 - e with dmax < 2^e, so that |w| 2^Fd < 2^62.
+template <typename R> struct SpItem;
+template <> struct __align__(8) SpItem<float> { float w; uint32_t xo; };
+template <> struct __align__(16) SpItem<double> { long long w; uint32_t xo, pad; };
+// Term groups (one case each): real terms (z_t, w_t) about a centre z_c,
+//   D(k) = (-1)^popc(k & z_c) sum_t w_t (-1)^popc(k & y_t), y_t = z_t ^ z_c
+// (a paired group: the kept terms doubled, and zero unless p0, the parity of
+// k & delta against neg, is zero).  The terms whose y lies within one of the
+// index ranges above are summed into tables over that range (of the source
+// index, x folded in), in fixed point: fa, fb, fc; those with y among the
+// tile's bits are summed once per tile (hy, hw; the constant f0 with them);
+// the others stay a list (ry over all bits, rw).  Integer sums, so their
+// order does not matter.
+template <typename R>
+struct __align__(16) SpTab {
+  using W = typename SpWeight<R>::T;
+  W fa[32], fb[16], fc[16];
+  uint32_t xo, x, rb, re;
+};
+// The per-tile part of a term group: f0 and the terms [hb, he) of hy, hw.
+template <typename R>
+struct __align__(8) SpTabTile {
+  typename SpWeight<R>::T f0;
+  uint32_t hb, he;
+};
+// A piece of the scatter kernel's work: nsub heads from sub0 (kind 0: LUT
+// cases, 1: term groups, the first in slot tab0), the groups sub0 ..
+// sub0 + nsub - 1 of the term lists (kind 2), or as many terms of the diagonal
+// group (kind 3: real, 4: imaginary), taken against span chunks of 32 source
+// amplitudes per unit.
+struct __align__(16) SpPiece {
+  uint32_t xhi, sub0;
+  uint16_t nsub, span;
+  uint16_t kind, tab0;
+};
+// A term-list group (imaginary weights, or terms that no centre gathers):
+// real terms [tb, tm), imaginary [tm, te); delta and neg as in TiledGroup.
+struct SpListGroup {
+  uint32_t x, tb, tm, te, delta, neg;
+};
+// The scatter kernel's tables (n_pieces = 0: none).
+struct SpTables {
+  int n_pieces = 0;
+  uint32_t n_sub = 0, n_tab = 0;    // heads; term groups in table form
+  const SpPiece* piece = nullptr;
+  const SpHead* head = nullptr;
+  const uint4* base = nullptr;      // per head
+  const uint4* hi = nullptr;        // hi[j n_sub + q]: head q, bit kSpLB + j of k
+  const uint4* fix = nullptr;       // per head: the cases whose p0, p1, p2 do not depend on k's low kSpLB bits
+  const void* item = nullptr;       // kSpCases SpItem<R> per head
+  const void* tab = nullptr;        // SpTab<R> per term group
+  const void* tile = nullptr;       // SpTabTile<R> per term group
+  const uint32_t* hy = nullptr;     // tile-bit terms (masks over the tile number) and weights
+  const void* hw = nullptr;
+  const uint32_t* ry = nullptr;     // list terms of the term groups and weights
+  const void* rw = nullptr;
+  const SpListGroup* list = nullptr;
+  const uint32_t* lz = nullptr;     // their terms: masks, weights (complex64: float, complex128: round(w 2^Fd))
+  const void* lw = nullptr;
+  float tscale = 1.f;               // 2^-Ft
+  double wscale = 1.0;              // 2^(63 - Fd): takes an amplitude scaled by 2^F to the integer whose product
+                                    // with a weight, shifted right by 63, is the product at 2^F
+  // the diagonal group and the identity (mask 0), weights as round(w 2^Fg),
+  // Fg = 62 - e with their sum of magnitudes < 2^e, and 2^(63 - Fg)
+  const uint32_t* dz = nullptr;
+  const long long* dq = nullptr;
+  double dscale = 1.0;
+};
+
 // Nonzero-amplitude list carried through a tracked chain of Taylor or
 // adjoint steps (LUT pools, n >= 8): the first entries of list hold every
 // nonzero amplitude index of the chain's state(s) (and possibly indices whose
@@ -271,14 +362,7 @@ struct DevTables {
   int n_pieces = 0;
   const uint8_t* tblob = nullptr;
   const TiledPiece* tpiece = nullptr;
-  const uint32_t* tporder = nullptr;   // piece indices by descending blob size
-  // complex128: the blobs' LUT entries and term-list weights as 64-bit
-  // fixed-point integers round(w 2^Fd), each at its value's offset in tblob
-  // (elsewhere zero), Fd = 62 - e with dmax < 2^e; and twscale = 2^(63 - Fd),
-  // the factor that takes an amplitude scaled by 2^F to the integer whose
-  // product with a weight, shifted right by 63, is the product at 2^F
-  const uint8_t* twfix = nullptr;
-  double twscale = 0.0;
+  SpTables sp;                  // the scatter kernel's form of the off-diagonal groups
   uint32_t* octmask = nullptr;
   uint32_t* tflags = nullptr;   // tiled form: one bit per tile (scratch)
   // second mask of the same size, for the adjoint sweep (psi and lambda)
@@ -532,17 +616,17 @@ int tiled_apply_h(const DevTables& t, const LiveOctets& lv, int precision, int s
                   void* hpsi, double identity, double* partials, unsigned int* counter,
                   unsigned int* tile_counter, double* scal, int32_t* err, cudaStream_t st);
 
-// Pieces the scatter kernel takes (two bytes of shared memory each); a
+// Pieces the scatter kernel takes (four bytes of shared memory each); a
 // problem with more keeps every state on the staged kernel.
-constexpr int kSpMaxPieces = 4096;
+constexpr int kSpMaxPieces = 8192;
+constexpr uint32_t kSpMaxTab = 2048;   // term groups in table form (shared memory per tile)
 
 // Arguments of the scatter kernel (apply_sparse.cu); see sparse_apply_h.
 template <typename R>
 struct SparseArgs {
-  const uint8_t* blob;
-  const TiledPiece* piece;
-  const uint32_t* porder;       // pieces by descending blob size (work units are numbered in this order)
-  int n_pieces, n;
+  SpTables sp;
+  bool base_smem;               // the heads' tile words fit in shared memory
+  int n;
   const C_t<R>* psi;
   C_t<R>* out;
   const uint32_t* mask;
@@ -553,16 +637,11 @@ struct SparseArgs {
   const unsigned long long* amax;   // max(|Re|, |Im|) of the listed amplitudes (double bits)
   double hbound;                // DevTables::hbound
   double dmax;                  // DevTables::dmax
-  const uint8_t* wfix;          // DevTables::twfix (complex128)
-  double wscale;                // DevTables::twscale (complex128)
   uint32_t parts;               // blocks per output tile (>= 1; > 1 needs gacc, tdone)
   unsigned long long* gacc;     // LiveOctets::gacc
   unsigned int* tdone;          // LiveOctets::tdone
   uint32_t max_amps;            // the kernel runs only when *alen <= max_amps (<= acap)
   uint32_t n_offdiag;           // off-diagonal groups (LUT and term-list): products per accumulator word
-  const uint32_t* dz;
-  const R* dw;
-  int nd, nd_mid;
   double identity;
   double* partials;
   unsigned int* counter;

@@ -1863,6 +1863,436 @@ PairedTerms<R> paired_terms(const std::vector<uint32_t>& tz, const std::vector<R
   return out;
 }
 
+// The scatter kernel's tables (SpTables) of the off-diagonal groups: hl in
+// LUT form, (gx, goff, gmid, tz, tw) as term lists; (dz, dw) the diagonal
+// group (real terms, then from nd_mid imaginary ones).  A high pattern's sub-blocks are cut into pieces of up to 8;
+// pieces are numbered by descending cost of a unit, so that the units left
+// at the end of a tile are short ones.  More pieces than kSpMaxPieces: no
+// scatter form.
+template <typename R>
+int build_scatter(int n, const std::vector<HLut<R>>& hl, const std::vector<uint32_t>& gx,
+                  const std::vector<int32_t>& goff, const std::vector<int32_t>& gmid, const std::vector<uint32_t>& tz,
+                  const std::vector<R>& tw, const std::vector<uint32_t>& dz, const std::vector<R>& dw, int nd_mid,
+                  double identity, DeviceTables& d, size_t& bytes) {
+  using W = typename SpWeight<R>::T;
+  constexpr uint32_t kLow = kSpTile - 1u;
+  const int nhi = std::max(0, n - kSpLB);
+  auto log2_above = [](double v) {   // e with |v| < 2^e
+    int e = 0;
+    if (v > 0.0) std::frexp(v, &e);
+    return e;
+  };
+  const int fd = 62 - log2_above(d.t.dmax);   // complex128 weights
+  SpTables T;
+  std::vector<SpHead> head;
+  std::vector<uint4> base;
+  std::vector<std::vector<uint4>> hi(nhi);
+  struct Costed {
+    SpPiece p;
+    uint32_t cost;
+  };
+  std::vector<Costed> pieces;
+  // a case under construction: the parities (masks over k and constants) that
+  // are zero where it applies, and its sign's
+  struct Case {
+    uint32_t x = 0, nc = 0, m[3] = {0, 0, 0}, e[3] = {0, 0, 0}, z = 0, ze = 0;
+    SpItem<R> it{};
+    uint32_t fixed() const {   // key: the conditions that do not depend on the low bits
+      uint32_t h = 0;
+      for (uint32_t q = 0; q < nc; ++q)
+        if (!(m[q] & kLow)) h ^= (m[q] >> kSpLB) * 0x9E3779B1u;
+      return h;
+    }
+    // The conditions in echelon form over the low bits: as many of them as
+    // possible depend on the tile number alone, which decides them for the
+    // whole tile.  False: never satisfied.
+    bool reduce() {
+      uint32_t done = 0;
+      for (int b = 0; b < kSpLB; ++b) {
+        uint32_t p = done;
+        while (p < nc && !((m[p] >> b) & 1u)) ++p;
+        if (p == nc) continue;
+        std::swap(m[done], m[p]);
+        std::swap(e[done], e[p]);
+        for (uint32_t q = 0; q < nc; ++q)
+          if (q != done && ((m[q] >> b) & 1u)) {
+            m[q] ^= m[done];
+            e[q] ^= e[done];
+          }
+        ++done;
+      }
+      uint32_t keep = 0;
+      for (uint32_t q = 0; q < nc; ++q) {
+        if (m[q]) {
+          m[keep] = m[q];
+          e[keep++] = e[q];
+        } else if (e[q]) {
+          return false;
+        }
+      }
+      nc = keep;
+      return true;
+    }
+  };
+  std::vector<uint4> fixm;
+  std::vector<SpItem<R>> items;
+  // Heads of 32 cases from cs[i, j) (one high pattern).
+  auto push_heads = [&](const std::vector<Case>& cs, size_t i, size_t j) {
+    for (; i < j; i += kSpCases) {
+      uint32_t bit[32][4] = {{0}};   // the words of a single bit of k
+      uint32_t c0[4] = {0, 0, 0, 0}, fx[3] = {0, 0, 0};
+      for (int g = 0; g < kSpCases; ++g) {
+        const uint32_t at = 0x80000000u >> g;
+        SpItem<R> it;
+        std::memset(&it, 0, sizeof(it));
+        if (i + g < j) {
+          const Case& c = cs[i + g];
+          it = c.it;
+          it.xo = 4u * (c.x & kLow);
+          for (uint32_t q = 0; q < 4; ++q) {
+            const uint32_t m = q == 3 ? c.z : q < c.nc ? c.m[q] : 0u, e = q == 3 ? c.ze : q < c.nc ? c.e[q] : 0u;
+            for (int b = 0; b < 32; ++b)
+              if ((m >> b) & 1u) bit[b][q] |= at;
+            if (((uint32_t)parity32(c.x & kLow & m) ^ e) & 1u) c0[q] |= at;
+            if (q < 3 && !(m & kLow)) fx[q] |= at;
+          }
+        } else {
+          c0[0] |= at;   // never applies
+          fx[0] |= at;
+        }
+        items.push_back(it);
+      }
+      auto word = [&](const uint32_t (&w)[4]) { return make_uint4(w[0], w[1], w[2], w[3]); };
+      auto fill = [&](uint4* t, int size, int from) {
+        t[0] = make_uint4(0u, 0u, 0u, 0u);
+        for (int v = 1; v < size; ++v) {
+          const uint4 a = t[v & (v - 1)], b = word(bit[from + __builtin_ctz(v)]);
+          t[v] = make_uint4(a.x ^ b.x, a.y ^ b.y, a.z ^ b.z, a.w ^ b.w);
+        }
+      };
+      SpHead h;
+      fill(h.ta, 32, 0);
+      fill(h.tb, 16, 5);
+      fill(h.tc, 16, 9);
+      head.push_back(h);
+      base.push_back(word(c0));
+      fixm.push_back(make_uint4(fx[0], fx[1], fx[2], 0u));
+      for (int b = 0; b < nhi; ++b) hi[b].push_back(word(bit[kSpLB + b]));
+    }
+  };
+  auto push_pieces = [&](uint32_t xhi, uint32_t s0, uint32_t s1, uint32_t kind, uint32_t max_sub, uint32_t each,
+                         uint32_t tab0) {
+    for (; s0 < s1; s0 += max_sub) {
+      Costed c;
+      std::memset(&c, 0, sizeof(c));
+      c.p.xhi = xhi;
+      c.p.sub0 = s0;
+      c.p.nsub = (uint16_t)std::min(max_sub, s1 - s0);
+      c.p.span = (uint16_t)(kind >= 2u ? 1u : std::max(1u, 4u / c.p.nsub));
+      c.p.kind = (uint16_t)kind;
+      c.p.tab0 = (uint16_t)tab0;
+      c.cost = each * c.p.nsub * c.p.span;
+      pieces.push_back(c);
+      tab0 += kSpCases * max_sub;
+    }
+  };
+  // ---- LUT groups, split into cases
+  std::vector<Case> cs;
+  for (const HLut<R>& L : hl) {
+    const uint32_t v[3] = {L.v0, L.v1, L.v2};
+    uint32_t left = 0;   // codes that occur, have a nonzero weight and are not covered yet
+    for (uint32_t c = 0; c < 8; ++c) {
+      bool occurs = true;
+      for (int q = 0; q < 3; ++q) occurs = occurs && (v[q] || !((c >> q) & 1u));
+      if (occurs && L.lut16[c] != R(0)) left |= 1u << c;
+    }
+    auto dot = [](uint32_t a, uint32_t b) { return (uint32_t)parity32(a & b); };
+    while (left) {
+      // the largest affine subspace o + span(d1, d2, ..) of the codes left on
+      // which |weight| is one value and the sign is affine
+      static const uint32_t kSpans[16][3] = {{1, 2, 4}, {1, 2, 0}, {1, 4, 0}, {2, 4, 0}, {1, 6, 0}, {2, 5, 0},
+                                             {4, 3, 0}, {3, 5, 0}, {1, 0, 0}, {2, 0, 0}, {3, 0, 0}, {4, 0, 0},
+                                             {5, 0, 0}, {6, 0, 0}, {7, 0, 0}, {0, 0, 0}};
+      bool found = false;
+      for (int k = 0; k < 16 && !found; ++k)
+        for (uint32_t o = 0; o < 8 && !found; ++o) {
+          const uint32_t* dv = kSpans[k];
+          const int dim = (dv[0] != 0) + (dv[1] != 0) + (dv[2] != 0);
+          uint32_t codes = 0, lin = 0;
+          bool ok = (left >> o) & 1u;
+          // sign: sigma(o + sum a_i d_i) = sigma(o) + sum a_i s_i
+          for (int a = 0; a < (1 << dim) && ok; ++a) {
+            uint32_t c = o, s = L.lut16[o] < R(0);
+            for (int q = 0; q < dim; ++q)
+              if ((a >> q) & 1) {
+                c ^= dv[q];
+                s ^= (uint32_t)((L.lut16[o ^ dv[q]] < R(0)) != (L.lut16[o] < R(0)));
+              }
+            ok = ((left >> c) & 1u) &&
+                 (a == 0 || (std::fabs((double)L.lut16[c]) == std::fabs((double)L.lut16[o]) &&
+                             (uint32_t)(L.lut16[c] < R(0)) == s));
+            codes |= 1u << c;
+          }
+          if (!ok) continue;
+          // a functional l with l . d_i = s_i gives the sign's linear part
+          bool have = false;
+          for (uint32_t l = 0; l < 8 && !have; ++l) {
+            have = true;
+            for (int q = 0; q < dim; ++q)
+              have = have && dot(l, dv[q]) == (uint32_t)((L.lut16[o ^ dv[q]] < R(0)) != (L.lut16[o] < R(0)));
+            if (have) lin = l;
+          }
+          Case c;
+          c.x = L.x;
+          // conditions: functionals that vanish on the directions, values as at o
+          uint32_t basis[3], nb = 0;
+          for (uint32_t f = 1; f < 8; ++f) {
+            bool van = true;
+            for (int q = 0; q < dim; ++q) van = van && dot(f, dv[q]) == 0u;
+            bool indep = van;
+            for (uint32_t m = 1; m < (1u << nb) && indep; ++m) {
+              uint32_t t = 0;
+              for (uint32_t q = 0; q < nb; ++q)
+                if ((m >> q) & 1u) t ^= basis[q];
+              indep = t != f;
+            }
+            if (indep && nb < 3) basis[nb++] = f;
+          }
+          auto mask = [&](uint32_t f) { return ((f & 1u) ? v[0] : 0u) ^ ((f & 2u) ? v[1] : 0u) ^ ((f & 4u) ? v[2] : 0u); };
+          for (uint32_t q = 0; q < nb; ++q) {
+            c.m[c.nc] = mask(basis[q]);
+            c.e[c.nc++] = dot(basis[q], o);
+          }
+          c.z = L.z0 ^ mask(lin);
+          c.ze = (uint32_t)(L.lut16[o] < R(0)) ^ dot(lin, o);
+          const double av = std::fabs((double)L.lut16[o]);
+          if constexpr (sizeof(R) == 4) c.it.w = (float)av;
+          else c.it.w = std::llround(std::ldexp(av, fd));
+          if (c.it.w != 0 && c.reduce()) cs.push_back(c);
+          left &= ~codes;
+          found = true;
+        }
+    }
+  }
+  std::stable_sort(cs.begin(), cs.end(), [](const Case& p, const Case& q) {
+    const uint32_t a = p.x >> kSpLB, b = q.x >> kSpLB;
+    return a != b ? a < b : p.fixed() < q.fixed();
+  });
+  for (size_t i = 0; i < cs.size();) {
+    const uint32_t xhi = cs[i].x >> kSpLB, first = (uint32_t)head.size();
+    size_t e = i;
+    while (e < cs.size() && (cs[e].x >> kSpLB) == xhi) ++e;
+    push_heads(cs, i, e);
+    push_pieces(xhi, first, (uint32_t)head.size(), 0u, 4u, 100u, 0u);
+    i = e;
+  }
+  // ---- term groups: those with real terms around a centre that at least
+  // half of them lie within one index range of, as tables; the others as
+  // lists.  The centre is the z of the term (among the first 64) that gathers
+  // most.
+  const uint32_t ranges[4] = {0x1Fu, 0x1E0u, 0x1E00u, ~kLow};
+  auto range_of = [&](uint32_t y) {   // -1: none
+    for (int q = 0; q < 4; ++q)
+      if ((y & ~ranges[q]) == 0u) return q;
+    return -1;
+  };
+  struct TabGroup {
+    uint32_t x, zc, delta, neg;
+    std::vector<uint32_t> y;
+    std::vector<double> w;
+  };
+  std::vector<TabGroup> tabs;
+  std::vector<SpListGroup> list;
+  std::vector<uint32_t> lz;
+  std::vector<double> lw;
+  std::vector<uint32_t> list_hi;
+  double tmax = 0.0;   // the largest sum of |w| of a table group
+  for (size_t g = 0; g < gx.size(); ++g) {
+    const auto pr = paired_terms<R>(tz, tw, goff[g], gmid[g], goff[g + 1]);
+    std::vector<uint32_t> z;
+    std::vector<double> w;
+    const bool real = gmid[g] == goff[g + 1];
+    if (pr.delta) {
+      z = pr.z;
+      w.assign(pr.w.begin(), pr.w.end());
+    } else {
+      z.assign(tz.begin() + goff[g], tz.begin() + goff[g + 1]);
+      w.assign(tw.begin() + goff[g], tw.begin() + goff[g + 1]);
+    }
+    size_t best = 0, at = 0;
+    if (real)
+      for (size_t c = 0; c < std::min<size_t>(64, z.size()); ++c) {
+        size_t in = 0;
+        for (uint32_t zt : z) in += range_of(zt ^ z[c]) >= 0;
+        if (in > best) {
+          best = in;
+          at = c;
+        }
+      }
+    if (real && 2 * best >= z.size() && !z.empty() && tabs.size() < kSpMaxTab) {
+      TabGroup t{gx[g], z[at], pr.delta, pr.neg, {}, {}};
+      double sum = 0.0;
+      for (size_t q = 0; q < z.size(); ++q) {
+        t.y.push_back(z[q] ^ z[at]);
+        t.w.push_back(pr.delta ? 2.0 * w[q] : w[q]);
+        sum += std::fabs(t.w.back());
+      }
+      tmax = std::max(tmax, sum);
+      tabs.push_back(std::move(t));
+    } else {
+      SpListGroup L;
+      L.x = gx[g];
+      L.tb = (uint32_t)lz.size();
+      L.tm = L.tb + (uint32_t)(pr.delta ? z.size() : (size_t)(gmid[g] - goff[g]));
+      L.te = L.tb + (uint32_t)z.size();
+      L.delta = pr.delta;
+      L.neg = pr.neg;
+      lz.insert(lz.end(), z.begin(), z.end());
+      lw.insert(lw.end(), w.begin(), w.end());
+      list.push_back(L);
+    }
+  }
+  const int ft = sizeof(R) == 4 ? 30 - log2_above(tmax) : fd;
+  auto fix = [&](double w) { return (W)std::llround(std::ldexp(w, ft)); };
+  std::stable_sort(tabs.begin(), tabs.end(),
+                   [](const TabGroup& a, const TabGroup& b) { return (a.x >> kSpLB) < (b.x >> kSpLB); });
+  std::vector<SpTab<R>> tab;
+  std::vector<SpTabTile<R>> tile;
+  std::vector<uint32_t> hy, ry;
+  std::vector<W> hw, rw;
+  for (size_t i = 0; i < tabs.size();) {
+    const uint32_t xhi = tabs[i].x >> kSpLB, first = (uint32_t)head.size();
+    const uint32_t tab0 = (uint32_t)tab.size();
+    std::vector<Case> tc;
+    for (; i < tabs.size() && (tabs[i].x >> kSpLB) == xhi; ++i) {
+      const TabGroup& t = tabs[i];
+      Case c;
+      c.x = t.x;
+      c.nc = t.delta ? 1u : 0u;
+      c.m[0] = t.delta;   // the factor is nonzero when the parity of k & delta equals neg
+      c.e[0] = t.delta ? t.neg : 0u;
+      c.z = t.zc;
+      tc.push_back(c);
+      SpTab<R> S;
+      std::memset(&S, 0, sizeof(S));
+      SpTabTile<R> tt;
+      std::memset(&tt, 0, sizeof(tt));
+      tt.hb = (uint32_t)hy.size();
+      S.xo = 4u * (t.x & kLow);
+      S.x = t.x;
+      S.rb = (uint32_t)ry.size();
+      for (size_t q = 0; q < t.y.size(); ++q) {
+        const uint32_t y = t.y[q];
+        const W wq = fix(t.w[q]);
+        const int rg = range_of(y);
+        auto spread = [&](W* f, int size, int from) {   // over the source bits
+          for (int v = 0; v < size; ++v) {
+            const uint32_t k = ((uint32_t)v << from) ^ (t.x & ranges[rg]);
+            f[v] += parity32(k & y) ? -wq : wq;
+          }
+        };
+        if (y == 0u) {
+          tt.f0 += wq;
+        } else if (rg == 0) {
+          spread(S.fa, 32, 0);
+        } else if (rg == 1) {
+          spread(S.fb, 16, 5);
+        } else if (rg == 2) {
+          spread(S.fc, 16, 9);
+        } else if (rg == 3) {
+          hy.push_back(y >> kSpLB);
+          hw.push_back(wq);
+        } else {
+          ry.push_back(y);
+          rw.push_back(wq);
+        }
+      }
+      S.re = (uint32_t)ry.size();
+      tt.he = (uint32_t)hy.size();
+      tab.push_back(S);
+      tile.push_back(tt);
+    }
+    push_heads(tc, 0, tc.size());
+    push_pieces(xhi, first, (uint32_t)head.size(), 1u, 1u, 300u, tab0);
+  }
+  // ---- list groups, up to 4 of one high pattern per piece
+  {
+    std::vector<int> lo(list.size());
+    for (size_t g = 0; g < lo.size(); ++g) lo[g] = (int)g;
+    std::stable_sort(lo.begin(), lo.end(), [&](int p, int q) { return (list[p].x >> kSpLB) < (list[q].x >> kSpLB); });
+    std::vector<SpListGroup> sorted;
+    for (int g : lo) sorted.push_back(list[g]);
+    list.swap(sorted);
+    for (size_t i = 0; i < list.size();) {
+      size_t e = i;
+      while (e < list.size() && (list[e].x >> kSpLB) == (list[i].x >> kSpLB)) ++e;
+      push_pieces(list[i].x >> kSpLB, (uint32_t)i, (uint32_t)e, 2u, 4u, 200u, 0u);
+      i = e;
+    }
+  }
+  // ---- the diagonal group and the identity: up to 64 terms per piece (a
+  // unit of all terms would be the longest of a tile by far)
+  std::vector<uint32_t> dzs;
+  std::vector<long long> dq;
+  double dsum = std::fabs(identity);
+  for (const R& w : dw) dsum += std::fabs((double)w);
+  const int fg = 62 - log2_above(dsum);
+  for (int imag = 0; imag < 2; ++imag) {
+    const uint32_t first = (uint32_t)dzs.size();
+    if (!imag && identity != 0.0) {
+      dzs.push_back(0u);
+      dq.push_back(std::llround(std::ldexp(identity, fg)));
+    }
+    for (int m = imag ? nd_mid : 0; m < (imag ? (int)dz.size() : nd_mid); ++m) {
+      dzs.push_back(dz[m]);
+      dq.push_back(std::llround(std::ldexp((double)dw[m], fg)));
+    }
+    push_pieces(0u, first, (uint32_t)dzs.size(), 3u + imag, 64u, 12u, 0u);
+  }
+  if (pieces.size() > (size_t)kSpMaxPieces) return GOCP_OK;
+  if (pieces.empty()) {   // H = 0: one piece without groups
+    Costed c;
+    std::memset(&c, 0, sizeof(c));
+    c.p.span = 1;
+    c.p.kind = 2;
+    pieces.push_back(c);
+  }
+  std::stable_sort(pieces.begin(), pieces.end(), [](const Costed& p, const Costed& q) { return p.cost > q.cost; });
+  std::vector<SpPiece> sp;
+  for (const Costed& c : pieces) sp.push_back(c.p);
+  std::vector<uint4> flat;
+  for (const auto& v : hi) flat.insert(flat.end(), v.begin(), v.end());
+  std::vector<R> lwr(lw.begin(), lw.end());
+  std::vector<long long> lwq;
+  for (double w : lw) lwq.push_back(std::llround(std::ldexp(w, fd)));
+  T.n_pieces = (int)sp.size();
+  T.n_sub = (uint32_t)head.size();
+  T.n_tab = (uint32_t)tile.size();
+  T.tscale = (float)std::ldexp(1.0, -ft);
+  T.wscale = std::ldexp(1.0, 63 - fd);
+  T.dscale = std::ldexp(1.0, 63 - fg);
+  int rc;
+  auto up = [&](auto& field, const auto& host) {
+    typename std::remove_const<typename std::remove_reference<decltype(host[0])>::type>::type* q = nullptr;
+    const int r = upload(d, &q, host, bytes);
+    field = q;
+    return r;
+  };
+  if ((rc = up(T.piece, sp)) || (rc = up(T.head, head)) || (rc = up(T.base, base)) || (rc = up(T.hi, flat)) ||
+      (rc = up(T.fix, fixm)) || (rc = up(T.item, items)) ||
+      (rc = up(T.dz, dzs)) || (rc = up(T.dq, dq)))
+    return rc;
+  if (!tab.empty() && ((rc = up(T.tab, tab)) || (rc = up(T.tile, tile)) || (rc = up(T.hy, hy)) ||
+                       (rc = up(T.hw, hw)) || (rc = up(T.ry, ry)) || (rc = up(T.rw, rw))))
+    return rc;
+  if (!list.empty()) {
+    if ((rc = up(T.list, list)) || (rc = up(T.lz, lz)) || (rc = sizeof(R) == 4 ? up(T.lw, lwr) : up(T.lw, lwq)))
+      return rc;
+  }
+  d.t.sp = T;
+  return GOCP_OK;
+}
+
 // Cuts the off-diagonal groups into the pieces of the tiled H psi kernel
 // (see TiledHead).  hl and the term-list groups come sorted by (x & 7, x),
 // an order each piece keeps.  Leaves t.n_pieces = 0 (the untiled kernel
@@ -1872,7 +2302,8 @@ template <typename R>
 int build_tiled(int n, const std::vector<HLut<R>>& hl, const std::vector<uint32_t>& gx,
                 const std::vector<int32_t>& goff, const std::vector<int32_t>& gmid,
                 const std::vector<uint64_t>& gbk, const std::vector<uint32_t>& tz,
-                const std::vector<R>& tw, DeviceTables& d, size_t& bytes) {
+                const std::vector<R>& tw, const std::vector<uint32_t>& dz, const std::vector<R>& dw, int nd_mid, double identity,
+                DeviceTables& d, size_t& bytes) {
   constexpr int LB = TiledBits<R>::LB;
   constexpr uint32_t octets = 1u << (LB - 3);
   static_assert(kTiledBlobBytes / sizeof(TiledGroup) < 4096, "run bounds of a piece fit 12 bits");
@@ -2003,68 +2434,24 @@ int build_tiled(int n, const std::vector<HLut<R>>& hl, const std::vector<uint32_
       pieces.push_back(pc);
     } while (li < ls.size() || ti < ts.size());
   }
-  // the scatter kernel numbers a tile's work units piece by piece in this
-  // order (costliest first), so that the units left at the end of a tile are
-  // short ones
-  std::vector<uint32_t> porder(pieces.size());
-  for (size_t i = 0; i < porder.size(); ++i) porder[i] = (uint32_t)i;
-  std::stable_sort(porder.begin(), porder.end(),
-                   [&](uint32_t a, uint32_t b) { return pieces[a].bytes > pieces[b].bytes; });
-  // complex128: the LUT entries and term weights again, as fixed-point
-  // integers round(w 2^Fd) at their own offsets (the scatter kernel forms
-  // its products in integers, see q_mul there).  Fd = 62 - e with
-  // dmax < 2^e, so that every |w| 2^Fd, and every group's sum of |w| 2^Fd,
-  // stays below 2^62.
-  std::vector<uint8_t> wfix;
-  int fd = 0;
-  if constexpr (sizeof(R) == 8) {
-    if (d.t.dmax > 0.0) {
-      int e;
-      std::frexp(d.t.dmax, &e);   // dmax < 2^e
-      fd = 62 - e;
-    }
-    auto put = [&](size_t at) {
-      double v;
-      std::memcpy(&v, blob.data() + at, sizeof(v));
-      const long long q = std::llround(std::ldexp(v, fd));
-      std::memcpy(wfix.data() + at, &q, sizeof(q));
-    };
-    wfix.assign(blob.size(), 0);
-    for (const TiledPiece& pc : pieces) {
-      TiledHead h;
-      std::memcpy(&h, blob.data() + pc.off, sizeof(h));
-      for (uint32_t g = 0; g < h.n_lut; ++g)
-        for (int c = 0; c < 16; ++c)
-          put(pc.off + sizeof(TiledHead) + g * sizeof(HLut<R>) + offsetof(HLut<R>, lut16) + c * sizeof(R));
-      for (uint32_t o = h.w_off; o + sizeof(R) <= pc.bytes; o += sizeof(R)) put(pc.off + o);
-    }
-  }
   uint8_t* dblob;
   TiledPiece* dpiece;
-  uint32_t* dporder;
   int rc;
-  if (!wfix.empty()) {
-    uint8_t* dw;
-    if ((rc = upload(d, &dw, wfix, bytes))) return rc;
-    d.t.twfix = dw;
-    d.t.twscale = std::ldexp(1.0, 63 - fd);
-  }
+  const size_t ntiles = n > kSpLB ? (size_t)1 << (n - kSpLB) : 1;   // scatter tiles
   if ((rc = upload(d, &dblob, blob, bytes)) || (rc = upload(d, &dpiece, pieces, bytes)) ||
-      (rc = upload(d, &dporder, porder, bytes)) ||
+      (rc = build_scatter<R>(n, hl, gx, goff, gmid, tz, tw, dz, dw, nd_mid, identity, d, bytes)) ||
       (rc = dalloc(d, &d.t.tflags, ((size_t)1 << (n - LB)) / 32 + 1, bytes)) ||
-      (rc = dalloc(d, &d.live.toff, ((size_t)1 << (n - LB)) + 1, bytes)) ||
+      (rc = dalloc(d, &d.live.toff, ntiles + 1, bytes)) ||
       (rc = dalloc(d, &d.live.aidx, (size_t)1 << (n - 2), bytes)) ||
       (rc = dalloc(d, reinterpret_cast<C_t<R>**>(&d.live.aval), (size_t)1 << (n - 2), bytes)) ||
       (rc = dalloc(d, &d.live.alen, 1, bytes)) || (rc = dalloc(d, &d.live.acounts, ((((size_t)1 << (n - 5)) + 255) / 256) + 1, bytes)) ||
       (rc = dalloc(d, &d.live.amax, 1, bytes)))
     return rc;
   d.live.acap = 1u << (n - 2);
-  // few output tiles (below 512: up to 21 qubits complex64, 20 complex128):
-  // global accumulators for the scatter kernel's blocks that share a tile,
-  // zero between calls
-  const size_t ntiles = (size_t)1 << (n - LB);
+  // few output tiles (below 512: up to 21 qubits): global accumulators for
+  // the scatter kernel's blocks that share a tile, zero between calls
   if (ntiles < 512) {
-    const size_t words = ntiles * (size_t)octets * 16u;
+    const size_t words = ntiles * (size_t)kSpTile * 2u;
     if ((rc = dalloc(d, &d.live.gacc, words, bytes)) || (rc = dalloc(d, &d.live.tdone, ntiles, bytes))) return rc;
     if ((rc = cuda_status(cudaMemset(d.live.gacc, 0, words * sizeof(unsigned long long)), "zero gacc")) ||
         (rc = cuda_status(cudaMemset(d.live.tdone, 0, ntiles * sizeof(unsigned int)), "zero tdone")))
@@ -2073,7 +2460,6 @@ int build_tiled(int n, const std::vector<HLut<R>>& hl, const std::vector<uint32_
   }
   d.t.tblob = dblob;
   d.t.tpiece = dpiece;
-  d.t.tporder = dporder;
   d.t.n_pieces = (int)pieces.size();
   return GOCP_OK;
 }
@@ -2252,7 +2638,7 @@ int upload_typed(Problem& p, DeviceTables& d, size_t& bytes, double* identity) {
     d.t.hbound = hb;
     d.t.dmax = dm;
   }
-  if ((rc = build_tiled<R>(p.n_qubits, hl, gx, goff, gmid, gbk, tz, tw, d, bytes))) return rc;
+  if ((rc = build_tiled<R>(p.n_qubits, hl, gx, goff, gmid, gbk, tz, tw, dz, dw, (int)dz_r.size(), ident, d, bytes))) return rc;
   // ---- pool
   const Pool& P = p.pool;
   const int M = P.size();
