@@ -197,13 +197,20 @@ int gocp_reference_state(const gocp_problem* p, void* psi, void* stream);
  * arrays per `mem`; ops must lie in [0, pool_size) (GOCP_EINVAL for host
  * arrays; device arrays are clamped and flagged, see gocp_device_errors).
  * n_ops may be 0.  A chain of several steps on a full-layout state of at
- * most 128 KiB runs in one thread block over shared memory (complex64 by
- * default); the environment variable GOCP_ONCHIP_CHAINS = "off" | "block" |
- * "all" selects the grid kernels only, the one-block form, or that and a
- * thread-block cluster's shared memory for states up to 2 MiB.  Larger
- * states run one launch per step, replayed as a CUDA graph whose steps are
- * joined by programmatic dependencies (GOCP_CHAIN_PDL=0: by full
- * completion).  Every form gives the same state bit for bit. */
+ * most 128 KiB (complex128: 11 qubits) runs in one thread block over shared
+ * memory; a chain on a larger state whose nonzero amplitudes are bounded (a
+ * problem built from integrals: the reference's determinants) runs in one
+ * launch whose blocks walk the list of nonzero amplitudes and wait for one
+ * another between steps (one cluster of 16 for short lists, every SM for longer
+ * ones; such a wait gives up after 2 s, or GOCP_CHAIN_WAIT_NS nanoseconds when
+ * that environment variable is set, see gocp_device_errors); other chains run
+ * one launch per step, replayed as a CUDA graph whose steps are joined by
+ * programmatic dependencies (GOCP_CHAIN_PDL=0: by full completion).  The
+ * environment variable GOCP_ONCHIP_CHAINS selects other forms: "off" a launch
+ * per step, "block" the one-block form where it fits, else that, "all" also a
+ * cluster's shared memory for states up to 2 MiB, "list" the list form
+ * for every problem (GOCP_LIST_SHARE caps the entries a block of it keeps in
+ * shared memory).  Every form gives the same state bit for bit. */
 int gocp_prepare_state(const gocp_problem* p, const int32_t* ops, const double* theta, int n_ops,
                        int mem, void* psi, void* stream);
 
@@ -286,7 +293,9 @@ int gocp_energy_static(const gocp_problem* p, const void* psi, void* hpsi, doubl
  * staging wait of the staged H psi kernel gave up (after 2 s, or after
  * GOCP_STAGE_WAIT_NS nanoseconds when that environment variable is set, at
  * once when it is 0; the H psi and energy of that call are then undefined,
- * later calls are not affected).  Synchronises `stream`. */
+ * later calls are not affected).  Bit 2: a wait between the blocks of a chain
+ * gave up (see gocp_prepare_state; the state, or dE, of that call is then
+ * undefined).  Synchronises `stream`. */
 int gocp_device_errors(const gocp_problem* p, int* flags, void* stream);
 
 /* ---------------------------------------------------------------- serving */

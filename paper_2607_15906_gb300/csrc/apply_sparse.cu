@@ -142,13 +142,13 @@ k_amp_count(const C_t<R>* __restrict__ psi, const C_t<R>* __restrict__ psi2, con
 
 // counts[0..nb) -> exclusive prefix sums in place; *total = the sum (when
 // set; and, when ring is set, the chain-list ring's base(slot) = the sum,
-// count(slot) = count(first) = 0); *amax = 0 when set.  One block of 1024
+// count(slot) = count(first) = 0); sync (when set) = 0; *amax = 0 when set.  One block of 1024
 // threads.  The sum reaches 2^32 only for a 32-qubit state with every
 // amplitude nonzero; it is stored saturated at 2^32 - 1 (above every list
 // capacity, so the list is not used), while every prefix, at most the sum
 // less the last block's count, fits 32 bits.
 __global__ void __launch_bounds__(1024)
-k_amp_scan(uint32_t* counts, uint32_t nb, uint32_t* total, uint32_t* ring, int slot, int first,
+k_amp_scan(uint32_t* counts, uint32_t nb, uint32_t* total, uint32_t* ring, uint32_t* sync, int slot, int first,
            unsigned long long* amax) {
   __shared__ uint32_t s[1024];
   __shared__ unsigned long long carry;
@@ -169,6 +169,8 @@ k_amp_scan(uint32_t* counts, uint32_t nb, uint32_t* total, uint32_t* ring, int s
     if (threadIdx.x == 0) carry += s[1023];
     __syncthreads();
   }
+  if (sync)
+    for (int w = threadIdx.x; w < kSyncWords; w += 1024) sync[w] = 0u;
   if (threadIdx.x == 0) {
     const uint32_t sum = carry > 0xffffffffull ? 0xffffffffu : (uint32_t)carry;
     if (total) *total = sum;
@@ -969,13 +971,13 @@ int amp_list(int precision, const void* psi, const uint32_t* mask, int n, const 
   if (precision == GOCP_C64) {
     const float2* p = reinterpret_cast<const float2*>(psi);
     k_amp_count<float><<<nb, kAmpBlock, 0, st>>>(p, nullptr, mask, words, lv.acounts);
-    k_amp_scan<<<1, 1024, 0, st>>>(lv.acounts, nb, lv.alen, nullptr, 0, 0, lv.amax);
+    k_amp_scan<<<1, 1024, 0, st>>>(lv.acounts, nb, lv.alen, nullptr, nullptr, 0, 0, lv.amax);
     k_amp_list<float><<<nb, kAmpBlock, 0, st>>>(p, nullptr, mask, words, lv.acounts, lv.aidx,
                                                 reinterpret_cast<float2*>(lv.aval), nullptr, lv.acap, lv.amax);
   } else {
     const double2* p = reinterpret_cast<const double2*>(psi);
     k_amp_count<double><<<nb, kAmpBlock, 0, st>>>(p, nullptr, mask, words, lv.acounts);
-    k_amp_scan<<<1, 1024, 0, st>>>(lv.acounts, nb, lv.alen, nullptr, 0, 0, lv.amax);
+    k_amp_scan<<<1, 1024, 0, st>>>(lv.acounts, nb, lv.alen, nullptr, nullptr, 0, 0, lv.amax);
     k_amp_list<double><<<nb, kAmpBlock, 0, st>>>(p, nullptr, mask, words, lv.acounts, lv.aidx,
                                                  reinterpret_cast<double2*>(lv.aval), nullptr, lv.acap, lv.amax);
   }
@@ -993,14 +995,14 @@ int chain_list(int precision, const void* psi, const void* lam, const uint32_t* 
     const float2* p = reinterpret_cast<const float2*>(psi);
     const float2* q = reinterpret_cast<const float2*>(lam);
     k_amp_count<float><<<nb, kAmpBlock, 0, st>>>(p, q, mask, words, counts);
-    k_amp_scan<<<1, 1024, 0, st>>>(counts, nb, nullptr, cl.cnt, slot, first, nullptr);
+    k_amp_scan<<<1, 1024, 0, st>>>(counts, nb, nullptr, cl.cnt, cl.sync, slot, first, nullptr);
     k_amp_list<float><<<nb, kAmpBlock, 0, st>>>(p, q, mask, words, counts, cl.list, nullptr, cl.amask, cl.cap,
                                                 nullptr);
   } else {
     const double2* p = reinterpret_cast<const double2*>(psi);
     const double2* q = reinterpret_cast<const double2*>(lam);
     k_amp_count<double><<<nb, kAmpBlock, 0, st>>>(p, q, mask, words, counts);
-    k_amp_scan<<<1, 1024, 0, st>>>(counts, nb, nullptr, cl.cnt, slot, first, nullptr);
+    k_amp_scan<<<1, 1024, 0, st>>>(counts, nb, nullptr, cl.cnt, cl.sync, slot, first, nullptr);
     k_amp_list<double><<<nb, kAmpBlock, 0, st>>>(p, q, mask, words, counts, cl.list, nullptr, cl.amask, cl.cap,
                                                  nullptr);
   }

@@ -233,6 +233,7 @@ int gocp_build(const gocp_build_args* a, gocp_problem** out) {
   p.n_qubits = 2 * a->n_orb;
   p.n_elec = a->n_elec;
   p.mapping = a->mapping;
+  p.terms_dropped = a->term_drop > 0.0;
   p.precision = a->precision;
   p.device = a->device;
   try {
@@ -640,6 +641,6 @@ int gocp_profile_read(int kind, int64_t* launches, double* total_ms) {
 const char* gocp_last_error(void) { return t_last_error.c_str(); }
 int64_t gocp_launch_count(void) { return g_launches.load(); }
 // The k_apply_h revision names the kernel that profiles/traffic.json was measured on.
-const char* gocp_version(void) { return "gocp-gb300 0.2 (sm_103a; k_apply_h_tiled=tiled-tma-r12; k_apply_h_sparse=scatter-cases-r19; chain=amp-list-ring-4; onchip=smem-chain-2; sector=pair-lists-csr-1; chains=graphs-pdl-2; grads=nonzero-amps-2)"; }
+const char* gocp_version(void) { return "gocp-gb300 0.2 (sm_103a; k_apply_h_tiled=tiled-tma-r12; k_apply_h_sparse=scatter-cases-r19; chain=amp-list-ring-4; list=coop-list-1; onchip=smem-chain-3; sector=pair-lists-csr-1; chains=graphs-pdl-2; grads=nonzero-amps-2)"; }
 
 }  // extern "C"

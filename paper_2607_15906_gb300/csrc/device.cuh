@@ -90,6 +90,14 @@ struct PairEnum {
   uint8_t nex, r, ncodes, log2cnt;
 };
 
+// The basis states k whose pair {k, k ^ x} a LUT-form generator touches, as a
+// test on k itself (either end): (k & S) == A or == B when two patterns of at
+// most six bits say it (S != 0; every excitation under Jordan-Wigner), else
+// bit phi(k) of codes.
+struct PairPat {
+  uint32_t S, A, B, codes;
+};
+
 __device__ __forceinline__ uint32_t enum_deposit(uint32_t c, uint32_t excl, int nex) {
   for (int e = 0; e < nex; ++e) {
     const uint32_t p = (excl >> (8 * e)) & 0xFFu;
@@ -305,10 +313,16 @@ __host__ __device__ constexpr int kRingBase(int i) { return 8 * i; }
 __host__ __device__ constexpr int kRingAdd(int i) { return 24 + 8 * i; }
 constexpr int kRingWords = 48;
 
+// Words of a list chain's synchronisation (ChainList::sync), each in its own
+// 32-byte sector: arrivals at the grid barrier, a flag, one inbox length per
+// block.
+constexpr int kSyncBar = 0, kSyncFull = 8, kSyncInbox = 16, kSyncWords = 16 + 8 * 256;
+
 struct ChainList {
   uint32_t* list = nullptr;
   uint32_t* amask = nullptr;
   uint32_t* cnt = nullptr;
+  uint32_t* sync = nullptr;   // zeroed where a chain's initial list is written
   uint32_t cap = 0;
 };
 
@@ -407,6 +421,7 @@ struct DevTables {
   bool pool_lut = false;
   const void* plut = nullptr;
   const PairEnum* penum = nullptr;
+  const PairPat* ppat = nullptr;
   uint32_t penum_max = 0;   // largest touched-pair count of any generator
   ChainList cl;             // tracked chains (list == nullptr: none)
 };

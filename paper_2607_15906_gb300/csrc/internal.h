@@ -130,6 +130,7 @@ struct Problem {
   size_t device_bytes = 0;
   // sector layout (GOCP_BUILD_SECTOR): states hold the D determinants with
   // n_alpha / n_beta electrons
+  bool terms_dropped = false;   // built with term_drop > 0: H may not conserve the electron counts exactly
   bool sector = false;
   int n_alpha = 0, n_beta = 0;
   int64_t sector_dim = 0;

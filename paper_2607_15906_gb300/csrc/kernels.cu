@@ -47,6 +47,13 @@ constexpr int kItemBlocksPerSm = 2;  // batched stages: blocks per item per SM
 #define GOCP_APPLY_MIN_BLOCKS_C64 4
 #endif
 
+// List chains (k_chain_list).
+constexpr uint64_t kListMaxAny = 65536, kListClusterC64 = 8192, kListClusterC128 = 2048;   // list_chain_blocks
+constexpr int kListMaxBlocks = 256;
+// Entries of the list and inbox buffers: a quarter of the state, 65,536 at
+// least (the inboxes of small states need room beyond their even share).
+uint32_t list_room(int n) { return std::max(1u << (n - 2), 65536u); }
+
 struct DeviceTables {
   DevTables t;
   int sm_count = 0;
@@ -68,6 +75,7 @@ struct DeviceTables {
   // kernel (n >= 8)
   LiveOctets live;
   uint32_t* chain_counts = nullptr;   // per-block counts of chain_list
+  uint32_t* chain_inbox = nullptr;    // list_room(n) entries (live.aidx where there is one)
   double* dpart = nullptr;            // stage_cap x adjoint_grid partials of dE/dtheta
 };
 
@@ -126,6 +134,8 @@ k_setup(C_t<R>* psi, int n, uint64_t index, const double* theta, int n_ops, doub
         cl.cnt[kRingAdd(2)] = 0u;
         cl.cnt[kRingAdd(0)] = 0u;
       }
+      if (blockIdx.x == 0)
+        for (int w = threadIdx.x; w < kSyncWords; w += kThreads) cl.sync[w] = 0u;
     }
   }
 }
@@ -749,7 +759,7 @@ k_taylor5(DevTables tb, const int32_t* ops, const double* coefs, int j, C_t<R>* 
 // pair marks both of its octets.
 // p1, p2 / q1, q2: the psi / lambda amplitudes of b and b ^ x.
 template <typename R>
-__device__ __forceinline__ double adjoint_pair_at(const LutDev<R>& L, const R (&c)[6], uint32_t b, uint32_t ph,
+__device__ __forceinline__ R adjoint_pair_at(const LutDev<R>& L, const R (&c)[6], uint32_t b, uint32_t ph,
                                                   C_t<R>* p1, C_t<R>* p2, C_t<R>* q1p, C_t<R>* q2p,
                                                   C_t<R> (&out)[4]) {
   const uint32_t phx = L.fx & 7u, sgx = (L.fx >> 3) & 1u;
@@ -768,8 +778,8 @@ __device__ __forceinline__ double adjoint_pair_at(const LutDev<R>& L, const R (&
   const C_t<R> t1 = cadd<R>(cscale<R>(q1, cd), cscale<R>(q2, cc * d1));
   const C_t<R> t2 = cadd<R>(cscale<R>(q2, cd), cscale<R>(q1, cc * d2));
   const C_t<R> l1v = *q1p, l2v = *q2p;
-  // the pair's term of 2 Re<lambda|T' psi>, formed in R (one conversion)
-  const double v = 2.0 * (double)(l1v.x * t1.x + l1v.y * t1.y + l2v.x * t2.x + l2v.y * t2.y);
+  // the pair's term of Re<lambda|T' psi>, formed in R (the caller doubles it)
+  const R v = l1v.x * t1.x + l1v.y * t1.y + l2v.x * t2.x + l2v.y * t2.y;
   out[0] = q1;
   out[1] = q2;
   out[2] = cadd<R>(cscale<R>(l1v, cc), cscale<R>(l2v, sd2));
@@ -785,7 +795,7 @@ template <typename R>
 __device__ __forceinline__ double adjoint_pair(const LutDev<R>& L, const R (&c)[6], uint32_t b, uint32_t ph,
                                                C_t<R>* psi, C_t<R>* lam, C_t<R> (&out)[4]) {
   const uint32_t b2 = b ^ L.x;
-  return adjoint_pair_at<R>(L, c, b, ph, psi + b, psi + b2, lam + b, lam + b2, out);
+  return 2.0 * (double)adjoint_pair_at<R>(L, c, b, ph, psi + b, psi + b2, lam + b, lam + b2, out);
 }
 
 // dpart set: each block writes its partial of dE_j to dpart[j nb + bid]
@@ -1763,6 +1773,38 @@ bool make_enum(const LutForm& f, uint32_t x, int n, PairEnum* out) {
   return true;
 }
 
+// Touched-pair test on a basis state (see PairPat).
+template <typename R>
+PairPat make_pat(const LutDev<R>& L) {
+  PairPat P;
+  std::memset(&P, 0, sizeof(P));
+  const uint32_t phx = L.fx & 7u;
+  for (uint32_t c = 0; c < 8; ++c)
+    if (L.lut[c] != R(0) || L.lut[c ^ phx] != R(0)) P.codes |= 1u << c;
+  const uint32_t S = L.v0 | L.v1 | L.v2;
+  const int bits = __builtin_popcount(S);
+  if (S == 0 || bits > 6) return P;
+  uint32_t found[2];
+  int cnt = 0;
+  for (uint32_t m = 0; m < (1u << bits) && cnt <= 2; ++m) {
+    uint32_t k = 0;   // m deposited into the bits of S
+    for (uint32_t s = S, b = 0; s; s &= s - 1u, ++b)
+      if ((m >> b) & 1u) k |= s & (~s + 1u);
+    const uint32_t ph = (uint32_t)parity32(k & L.v0) | ((uint32_t)parity32(k & L.v1) << 1) |
+                        ((uint32_t)parity32(k & L.v2) << 2);
+    if ((P.codes >> ph) & 1u) {
+      if (cnt < 2) found[cnt] = k;
+      ++cnt;
+    }
+  }
+  if (cnt == 1 || cnt == 2) {
+    P.S = S;
+    P.A = found[0];
+    P.B = found[cnt - 1];
+  }
+  return P;
+}
+
 // LUT descriptor of one H x-group for the octet layout of the H psi kernel.
 template <typename R>
 bool make_hlut(uint32_t x, const std::vector<uint32_t>& z, const std::vector<double>& w, HLut<R>* out) {
@@ -2271,24 +2313,40 @@ int build_scatter(int n, const std::vector<HLut<R>>& hl, const std::vector<uint3
   T.tscale = (float)std::ldexp(1.0, -ft);
   T.wscale = std::ldexp(1.0, 63 - fd);
   T.dscale = std::ldexp(1.0, 63 - fg);
-  int rc;
-  auto up = [&](auto& field, const auto& host) {
-    typename std::remove_const<typename std::remove_reference<decltype(host[0])>::type>::type* q = nullptr;
-    const int r = upload(d, &q, host, bytes);
-    field = q;
-    return r;
+  // one device buffer for all of it: an allocation and a copy each would cost
+  // a small problem's build more than its tables
+  std::vector<uint4> buf;
+  auto put = [&](const auto& host) {
+    const size_t at = buf.size(), sz = host.size() * sizeof(host[0]);
+    buf.resize(at + (sz + 15) / 16);
+    if (sz) std::memcpy(buf.data() + at, host.data(), sz);
+    return at;
   };
-  if ((rc = up(T.piece, sp)) || (rc = up(T.head, head)) || (rc = up(T.base, base)) || (rc = up(T.hi, flat)) ||
-      (rc = up(T.fix, fixm)) || (rc = up(T.item, items)) ||
-      (rc = up(T.dz, dzs)) || (rc = up(T.dq, dq)))
-    return rc;
-  if (!tab.empty() && ((rc = up(T.tab, tab)) || (rc = up(T.tile, tile)) || (rc = up(T.hy, hy)) ||
-                       (rc = up(T.hw, hw)) || (rc = up(T.ry, ry)) || (rc = up(T.rw, rw))))
-    return rc;
-  if (!list.empty()) {
-    if ((rc = up(T.list, list)) || (rc = up(T.lz, lz)) || (rc = sizeof(R) == 4 ? up(T.lw, lwr) : up(T.lw, lwq)))
-      return rc;
-  }
+  const size_t o_piece = put(sp), o_head = put(head), o_base = put(base), o_hi = put(flat), o_fix = put(fixm),
+               o_item = put(items), o_dz = put(dzs), o_dq = put(dq), o_tab = put(tab), o_tile = put(tile),
+               o_hy = put(hy), o_hw = put(hw), o_ry = put(ry), o_rw = put(rw), o_list = put(list), o_lz = put(lz),
+               o_lw = sizeof(R) == 4 ? put(lwr) : put(lwq);
+  uint4* dev = nullptr;
+  const int rc = upload(d, &dev, buf, bytes);
+  if (rc) return rc;
+  auto at = [&](auto& field, size_t o) { field = reinterpret_cast<typename std::remove_reference<decltype(field)>::type>(dev + o); };
+  at(T.piece, o_piece);
+  at(T.head, o_head);
+  at(T.base, o_base);
+  at(T.hi, o_hi);
+  at(T.fix, o_fix);
+  at(T.item, o_item);
+  at(T.dz, o_dz);
+  at(T.dq, o_dq);
+  at(T.tab, o_tab);
+  at(T.tile, o_tile);
+  at(T.hy, o_hy);
+  at(T.hw, o_hw);
+  at(T.ry, o_ry);
+  at(T.rw, o_rw);
+  at(T.list, o_list);
+  at(T.lz, o_lz);
+  at(T.lw, o_lw);
   d.t.sp = T;
   return GOCP_OK;
 }
@@ -2442,7 +2500,7 @@ int build_tiled(int n, const std::vector<HLut<R>>& hl, const std::vector<uint32_
       (rc = build_scatter<R>(n, hl, gx, goff, gmid, tz, tw, dz, dw, nd_mid, identity, d, bytes)) ||
       (rc = dalloc(d, &d.t.tflags, ((size_t)1 << (n - LB)) / 32 + 1, bytes)) ||
       (rc = dalloc(d, &d.live.toff, ntiles + 1, bytes)) ||
-      (rc = dalloc(d, &d.live.aidx, (size_t)1 << (n - 2), bytes)) ||
+      (rc = dalloc(d, &d.live.aidx, list_room(n), bytes)) ||
       (rc = dalloc(d, reinterpret_cast<C_t<R>**>(&d.live.aval), (size_t)1 << (n - 2), bytes)) ||
       (rc = dalloc(d, &d.live.alen, 1, bytes)) || (rc = dalloc(d, &d.live.acounts, ((((size_t)1 << (n - 5)) + 255) / 256) + 1, bytes)) ||
       (rc = dalloc(d, &d.live.amax, 1, bytes)))
@@ -2663,6 +2721,7 @@ int upload_typed(Problem& p, DeviceTables& d, size_t& bytes, double* identity) {
   poff.push_back((int32_t)pz.size());
   std::vector<LutDev<R>> pl(M);
   std::vector<PairEnum> pe(M);
+  std::vector<PairPat> pp(M);
   uint32_t pe_max = 0;
   bool all_lut = M > 0;
   for (int k = 0; k < M && all_lut; ++k) {
@@ -2683,6 +2742,7 @@ int upload_typed(Problem& p, DeviceTables& d, size_t& bytes, double* identity) {
         std::memset(&pe[k], 0, sizeof(PairEnum));
       }
       pe_max = std::max(pe_max, (uint32_t)pe[k].ncodes << pe[k].log2cnt);
+      pp[k] = make_pat<R>(pl[k]);
     }
   }
   for (int k = 0; k < M; ++k) porder[k] = k;
@@ -2709,7 +2769,15 @@ int upload_typed(Problem& p, DeviceTables& d, size_t& bytes, double* identity) {
   if (all_lut) {
     LutDev<R>* dpl = nullptr;
     PairEnum* dpe;
-    if ((rc = upload(d, &dpl, pl, bytes)) || (rc = upload(d, &dpe, pe, bytes))) return rc;
+    // the patterns follow the enumerations in one buffer
+    static_assert(sizeof(PairEnum) % alignof(PairPat) == 0, "patterns are aligned after the enumerations");
+    std::vector<uint8_t> buf(M * (sizeof(PairEnum) + sizeof(PairPat)));
+    std::memcpy(buf.data(), pe.data(), M * sizeof(PairEnum));
+    std::memcpy(buf.data() + M * sizeof(PairEnum), pp.data(), M * sizeof(PairPat));
+    uint8_t* dbuf = nullptr;
+    if ((rc = upload(d, &dpl, pl, bytes)) || (rc = upload(d, &dbuf, buf, bytes))) return rc;
+    dpe = reinterpret_cast<PairEnum*>(dbuf);
+    d.t.ppat = reinterpret_cast<const PairPat*>(dbuf + M * sizeof(PairEnum));
     d.t.plut = dpl;
     d.t.penum = dpe;
     d.t.penum_max = pe_max;
@@ -2816,10 +2884,13 @@ int upload_problem(Problem& p) {
     // chain list: a quarter of the state's indices at most, one amplitude-mask bit each
     const int n = p.n_qubits;
     const size_t nb = ((((size_t)1 << (n - 5)) + 255) / 256) + 1;
-    if ((rc = dalloc(*d, &d->t.cl.list, (size_t)1 << (n - 2), bytes)) ||
-        (rc = dalloc(*d, &d->t.cl.amask, (size_t)1 << (n - 5), bytes)) || (rc = dalloc(*d, &d->t.cl.cnt, kRingWords, bytes)) ||
+    d->chain_inbox = d->live.aidx;
+    if ((!d->chain_inbox && (rc = dalloc(*d, &d->chain_inbox, list_room(n), bytes))) ||
+        (rc = dalloc(*d, &d->t.cl.list, list_room(n), bytes)) ||
+        (rc = dalloc(*d, &d->t.cl.amask, (size_t)1 << (n - 5), bytes)) || (rc = dalloc(*d, &d->t.cl.cnt, kRingWords + kSyncWords, bytes)) ||
         (rc = dalloc(*d, &d->chain_counts, nb, bytes)))
       return rc;
+    d->t.cl.sync = d->t.cl.cnt + kRingWords;
     d->t.cl.cap = 1u << (n - 2);
   }
   int sm = 0;
@@ -2861,18 +2932,27 @@ void free_device(Problem& p) {
 }
 
 // Which on-chip chain forms may run: GOCP_ONCHIP_CHAINS = "all" (one block
-// and clusters), "block" (one block only), "off" (the grid kernels only);
-// default "block" for complex64 and "off" for complex128, whose FP64
-// arithmetic is better spread over every SM than held in a few.
+// and clusters), "block" (one block only), "off" (the grid kernels only).
+// "list": list chains only.  Unset: one block for complex64, and for
+// complex128 up to kSmemC128Qubits (40-operator energy_grad at 8 and 10 qubits 365 and 510 us
+// against 468 and 595 as list chains and 507 and 664 with a launch per step;
+// 460 against 441 at 12 qubits: FP64 arithmetic is better spread over SMs than
+// held in one), and list chains (list_chain_blocks).
 enum { kOnchipOff = 0, kOnchipBlock = 1, kOnchipAll = 2 };
-int onchip_mode(int precision) {
+int onchip_mode() {
   const char* e = std::getenv("GOCP_ONCHIP_CHAINS");
   if (e && *e) {
     if (!std::strcmp(e, "all")) return kOnchipAll;
     if (!std::strcmp(e, "block")) return kOnchipBlock;
     if (!std::strcmp(e, "off")) return kOnchipOff;
   }
-  return precision == GOCP_C64 ? kOnchipBlock : kOnchipOff;
+  return kOnchipBlock;
+}
+// Largest complex128 state the one-block forms take unless asked for.
+constexpr int kSmemC128Qubits = 11;
+bool onchip_is(const char* mode) {   // nullptr: unset
+  const char* e = std::getenv("GOCP_ONCHIP_CHAINS");
+  return e && *e ? mode && !std::strcmp(e, mode) : !mode;
 }
 
 // ---- chains in cluster shared memory (DSMEM)
@@ -2988,7 +3068,7 @@ __device__ void adjoint_chain_cluster_body(const DevTables& tb, const int32_t* o
       C_t<R>* l2 = cl.map_shared_rank(ml + o2, r2);
       if (cz<R>(*a1) && cz<R>(*a2) && cz<R>(*l1) && cz<R>(*l2)) continue;   // nothing to add, stays zero
       C_t<R> o[4];
-      v += adjoint_pair_at<R>(L, c, b, ph, a1, a2, l1, l2, o);
+      v += 2.0 * (double)adjoint_pair_at<R>(L, c, b, ph, a1, a2, l1, l2, o);
     }
     const double w = __any_sync(0xffffffffu, v != 0.0) ? warp_sum(v) : 0.0;
     if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = w;
@@ -3041,12 +3121,384 @@ __global__ void __launch_bounds__(kSmemThreads, 1) k_stage_backward_cluster(cons
 // does or none fits.
 template <typename R>
 int chain_cluster_blocks(const DeviceTables& d, int states) {
-  if (!d.t.pool_lut || onchip_mode(sizeof(R) == 4 ? GOCP_C64 : GOCP_C128) < kOnchipAll) return 0;
+  if (!d.t.pool_lut || onchip_mode() < kOnchipAll) return 0;
   const uint64_t bytes = ((uint64_t)states << d.t.n) * sizeof(C_t<R>);
   if (bytes <= kSmemStateBytes) return 0;
   for (int c = 2; c <= kClusterMax; c *= 2)
     if (bytes <= (uint64_t)c * kSmemStateBytes && (1ull << d.t.n) % (uint64_t)c == 0) return c;
   return 0;
+}
+
+// ---- list chains
+//
+// A tracked chain over the nonzero amplitudes of its state(s) in one
+// cooperative launch.  The state stays in global memory (its lines in L2).
+// The list of nonzero amplitude indices is dealt out to the blocks, each
+// keeping its share in shared memory.  A step is
+//   A  each warp tests its entries against the operator (is the entry's pair
+//      touched: two compares of the bits the operator acts on, or the LUT
+//      code's parities) and packs the few that are into its own queue;
+//   B  the warp takes 32 queued entries at a time: membership bit and
+//      amplitudes are independent loads, then the same per-pair arithmetic as
+//      the one-launch-per-step kernels; an end that became nonzero joins the
+//      block's own share, or, while that is small, the inbox of a block chosen
+//      by its index (a chain starts from one entry: the inboxes spread its
+//      first descendants evenly, and their descendants stay where they are,
+//      which spares them a round trip to L2);
+// and a grid barrier.  A of the next step needs shared memory only, so it runs
+// while the barrier completes; entries from the inbox are tested after it.
+//
+// What bounds a step is a chain of L2 round trips: the pair's loads, the
+// barrier's fence and arrival, its poll, the inbox.  A launch per step repeated
+// more of them (operator, descriptor, list length, list, membership, state)
+// behind its launch latency.  Measured: see list_chain_blocks.
+constexpr uint32_t kListSmem = 24576;    // entries of a block's share in shared memory; the rest are read in place
+constexpr uint32_t kListOwn = 64;        // share from which a block keeps its new entries
+constexpr uint32_t kListQueue = 512;     // queued entries per warp
+constexpr int kListChunk = 32;           // steps staged at a time
+constexpr int32_t kErrChainTimeout = 4;
+constexpr uint64_t kChainWaitNs = 2000000000ull;   // limit of a barrier wait: 2 s
+
+template <typename R>
+struct ListStep {
+  LutDev<R> L;
+  PairEnum E;
+  PairPat P;
+  R c[6];
+  int valid;
+};
+template <typename R>
+constexpr size_t list_smem() {
+  return 4u * kListSmem + 4u * kListQueue * (kSmemThreads / 32) + 2 * kListChunk * sizeof(ListStep<R>);
+}
+
+// dE_j partial sums: complex64 terms are summed as unevaluated pairs of floats
+// (TwoSum, about 48 bits: the FP64 pipe is narrow here), complex128 in FP64.
+struct PairSum {
+  float s, e;
+  __device__ __forceinline__ void add(float v) {
+    const float t = s + v, z = t - s;
+    e += (s - (t - z)) + (v - z);
+    s = t;
+  }
+  __device__ __forceinline__ void warp() {
+    for (int o = 16; o > 0; o >>= 1) {
+      const float s2 = __shfl_down_sync(0xffffffffu, s, o), e2 = __shfl_down_sync(0xffffffffu, e, o);
+      add(s2);
+      e += e2;
+    }
+  }
+  __device__ __forceinline__ bool any() const { return s != 0.f || e != 0.f; }
+  __device__ __forceinline__ double total() const { return (double)s + (double)e; }
+};
+struct DoubleSum {
+  double s;
+  __device__ __forceinline__ void add(double v) { s += v; }
+  __device__ __forceinline__ void warp() { s = warp_sum(s); }
+  __device__ __forceinline__ bool any() const { return !rzero<double>(s); }
+  __device__ __forceinline__ double total() const { return s; }
+};
+template <typename R> struct StepSum { using T = PairSum; };
+template <> struct StepSum<double> { using T = DoubleSum; };
+
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+__device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+
+__device__ __forceinline__ void red_release(uint32_t* p) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p) : "memory");
+}
+
+// BACK false: psi <- the chain applied to psi, starting from the list {ref}
+// (the reference state dev_setup wrote).  BACK true: the adjoint sweep over
+// psi and lam, from the list chain_list wrote (its length in ring slot
+// `slot`); dpart[j G + block] = the block's part of dE_j.  mask: octet mask of
+// psi (or psi and lam), kept valid.  inbox: seg entries per block; cap:
+// entries of a share in shared memory (at most kListSmem).  A list
+// that is incomplete, or an inbox that overflows, is given up for the
+// operator's enumerated pairs (full).  tb.cl.sync: the barrier's count, the
+// full flag and the inbox lengths, zero at the start.  CLUSTER: the blocks are
+// one thread-block cluster and take its hardware barrier; else the barrier is
+// a count in global memory whose wait gives up after wait_ns (recorded in err,
+// the results are then undefined).
+template <typename R, bool BACK, bool CLUSTER>
+__global__ void __launch_bounds__(kSmemThreads, 1)
+k_chain_list(DevTables tb, const int32_t* ops, const double* coefs, int n_ops, C_t<R>* psi, C_t<R>* lam,
+             uint32_t* mask, uint32_t ref, int slot, uint32_t* inbox, uint32_t seg, double* dpart, int32_t* err,
+             uint32_t cap, uint64_t wait_ns) {
+  using Sum = typename StepSum<R>::T;
+  extern __shared__ __align__(16) uint8_t cl_raw[];
+  uint32_t* list = reinterpret_cast<uint32_t*>(cl_raw);
+  uint32_t* queue = list + kListSmem;
+  ListStep<R>* sd = reinterpret_cast<ListStep<R>*>(queue + kListQueue * (kSmemThreads / 32));
+  __shared__ uint32_t s_in, s_full, s_n;   // inbox length; see full; entries of the share in list
+  __shared__ int s_abort;
+  __shared__ Sum s_sum[kSmemThreads / 32];
+  const uint32_t G = gridDim.x, rank = blockIdx.x;
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, lt = (1u << lane) - 1u;
+  constexpr uint32_t kW = kSmemThreads / 32;
+  uint32_t* wq = queue + kListQueue * warp;
+  uint32_t* bar = tb.cl.sync + kSyncBar;
+  uint32_t* full_flag = tb.cl.sync + kSyncFull;
+  uint32_t* in_lens = tb.cl.sync + kSyncInbox;   // + 8 rank
+  const uint32_t* mine_in = inbox + (size_t)rank * seg;
+  // ---- the share: list[0 .. n_list) (initial entries, own and inbox ones),
+  // then what found no room there: initial entries [cap, n_first) (BACK:
+  // entry e of the initial list is the block's when (e / 32) mod G is its
+  // number) and inbox entries from in_base on, read in place
+  uint32_t n_first = 0, full = 0;
+  if constexpr (BACK) {
+    const uint32_t total = tb.cl.cnt[kRingBase(slot)] + tb.cl.cnt[kRingAdd(slot)];
+    if (total > tb.cl.cap) {
+      full = 1u;
+    } else {
+      const uint32_t chunks = (total + 31u) / 32u;
+      const uint32_t own = rank < chunks ? (chunks - rank + G - 1u) / G : 0u;
+      n_first = 32u * own;   // less what the list's last chunk lacks, in its owner's last
+      if (own && (chunks - 1u) % G == rank) n_first -= 32u * chunks - total;
+      for (uint32_t i = threadIdx.x; i < min(n_first, cap); i += kSmemThreads)
+        list[i] = tb.cl.list[((i >> 5) * G + rank) * 32u + (i & 31u)];
+    }
+  } else if (rank == 0) {
+    n_first = 1u;
+    if (threadIdx.x == 0) list[0] = ref;
+  }
+  uint32_t n_list = min(n_first, cap), in_base = 0u, in_len = 0u;
+  const uint32_t n_far = n_first - n_list;
+  if (threadIdx.x == 0) {
+    s_n = n_list;
+    s_in = 0u;
+    s_full = full;
+    s_abort = 0;
+  }
+  auto entry = [&](uint32_t i) -> uint32_t {   // entry i of the share
+    if (i < n_list) return list[i];
+    i -= n_list;
+    if (i < n_far) {
+      const uint32_t q = cap + i;
+      return __ldcg(tb.cl.list + (((q >> 5) * G + rank) * 32u + (q & 31u)));
+    }
+    return __ldcg(mine_in + (in_base + i - n_far));
+  };
+  auto stage = [&](int i) {   // steps i .. i + kListChunk - 1 into their half of sd
+    for (int q = (int)warp; q < min(n_ops - i, kListChunk); q += (int)kW) {
+      const int jq = BACK ? n_ops - 1 - (i + q) : i + q, op = ops[jq];
+      ListStep<R>& D = sd[(i + q) % (2 * kListChunk)];
+      const bool ok = op >= 0 && op < tb.M;
+      if (lane == 0) D.valid = ok ? 1 : 0;
+      if (!ok) {
+        if (rank == 0 && lane == 0) atomicOr(err, 1);
+        continue;
+      }
+      copy_words(&D.L, ((const LutDev<R>*)tb.plut) + op);
+      copy_words(&D.E, tb.penum + op);
+      copy_words(&D.P, tb.ppat + op);
+      if (lane < 6) D.c[lane] = (R)coefs[6 * jq + lane];
+    }
+  };
+  stage(0);
+  __syncthreads();
+  uint32_t cnt = 0, at = 0;   // this warp's queue length; entries [0, at) of the share (by warp stride) tested
+  for (int i = 0; i < n_ops; ++i) {
+    const int j = BACK ? n_ops - 1 - i : i;
+    const ListStep<R>& D = sd[i % (2 * kListChunk)];
+    const LutDev<R>& L = D.L;
+    const PairPat P = D.P;
+    const bool walk = D.valid && !full;
+    auto test = [&](uint32_t e, bool on) {   // entry e of each lane (if on): queue the touched ones
+      const uint32_t k = on ? entry(e) : 0u;
+      bool hit;
+      if (P.S) {
+        const uint32_t t = k & P.S;
+        hit = t == P.A || t == P.B;
+      } else {
+        hit = (P.codes >> lut_phi(L, k)) & 1u;
+      }
+      hit = hit && on;
+      const uint32_t m = __ballot_sync(0xffffffffu, hit);
+      if (hit) wq[cnt + __popc(m & lt)] = k;
+      cnt += __popc(m);
+    };
+    // A: the entries known so far, as far as the queue has room
+    uint32_t n = n_list + n_far + (in_len - in_base);
+    cnt = 0;
+    at = warp * 32u;
+    if (walk)
+      for (; at < n && cnt <= kListQueue - 64u; at += kSmemThreads) test(at + lane, at + lane < n);
+    if (i > 0) {
+      // the barrier of the step before, then the inbox: its length and, in the
+      // same round trip, the first 32 entries it may have gained
+      if constexpr (CLUSTER) cluster_wait();
+      if (warp == 0) {
+        if (!CLUSTER && lane == 0) {
+          const uint32_t want = (uint32_t)i * G;
+          if (wait_ns == 0 || ld_acquire(bar) < want) {
+            uint64_t t0, t1;
+            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+            for (uint32_t spin = 0;; ++spin) {
+              if (wait_ns != 0 && ld_acquire(bar) >= want) break;
+              if (wait_ns == 0 || (spin & 1023u) == 1023u) {
+                asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
+                if (wait_ns == 0 || t1 - t0 > wait_ns) {
+                  atomicOr(err, kErrChainTimeout);
+                  s_abort = 1;
+                  break;
+                }
+              }
+            }
+          }
+        }
+        __syncwarp();
+        const uint32_t got = min(__ldcg(in_lens + 8u * rank), seg), over = __ldcg(full_flag);
+        const uint32_t q = in_len + lane, early = q < seg ? __ldcg(mine_in + q) : 0u;
+        if (n_far == 0u && in_base == in_len && q < got && n_list + lane < cap) list[n_list + lane] = early;
+        if (lane == 0) {
+          s_in = got;
+          if (over) s_full = 1u;
+        }
+      }
+      __syncthreads();
+      if (s_abort) return;
+      full = s_full;
+      if (s_in > in_len) {
+        // while the list has room (and nothing is read in place yet) the new
+        // entries join it; the first 32 are there already
+        const uint32_t more = s_in - in_len;
+        const uint32_t fit = n_far == 0u && in_base == in_len ? min(more, cap - n_list) : 0u;
+        if (fit > 32u) {
+          for (uint32_t q = 32u + threadIdx.x; q < fit; q += kSmemThreads) list[n_list + q] = __ldcg(mine_in + in_len + q);
+          __syncthreads();
+        }
+        const uint32_t old = n;
+        if (threadIdx.x == 0) s_n = n_list + fit;
+        n_list += fit;
+        in_base += fit;
+        in_len = s_in;
+        n = n_list + n_far + (in_len - in_base);
+        // entries [old, n): of a warp's row that A tested in part, the rest
+        if (walk && !full) {
+          const uint32_t row = old & ~31u;
+          if ((old & 31u) && (row / 32u) % kW == warp && at > row) test(row + lane, row + lane >= old && row + lane < n);
+        }
+        __syncthreads();   // s_n is set before anyone adds to it
+      }
+    }
+    // B
+    Sum sum{};
+    if (D.valid) {
+      R c[6];
+#pragma unroll
+      for (int m = 0; m < 6; ++m) c[m] = D.c[m];
+      const uint32_t x = L.x;
+      // new entries stay here once the share is large enough to be typical of
+      // the whole list, while list has room and is all of the share
+      const bool own = n_list >= kListOwn && n_list < cap && n == n_list;
+      auto pair = [&](uint32_t k) {   // one pair, by its entry k: `other` is its other end
+        const uint32_t other = k ^ x;
+        const bool base = !((k >> L.s) & 1u);
+        const uint32_t word = __ldcg(tb.cl.amask + (other >> 5));
+        const C_t<R> vk = __ldcg(psi + k), vo = __ldcg(psi + other);
+        C_t<R> lk, lo;
+        if constexpr (BACK) {
+          lk = __ldcg(lam + k);
+          lo = __ldcg(lam + other);
+        }
+        const bool listed = (word >> (other & 31u)) & 1u;
+        if (!base && listed) return;   // the base's entry computes the pair
+        const uint32_t b = base ? k : other, ph = lut_phi(L, b);
+        C_t<R> p1 = base ? vk : vo, p2 = base ? vo : vk;
+        bool nz;
+        if constexpr (BACK) {
+          C_t<R> q1 = base ? lk : lo, q2 = base ? lo : lk, o[4];
+          sum.add(adjoint_pair_at<R>(L, c, b, ph, &p1, &p2, &q1, &q2, o));
+          __stcg(lam + b, q1);
+          __stcg(lam + (b ^ x), q2);
+          const C_t<R> po = base ? p2 : p1, qo = base ? q2 : q1;
+          nz = !(rzero<R>(po.x) && rzero<R>(po.y) && rzero<R>(qo.x) && rzero<R>(qo.y));
+        } else {
+          C_t<R> o1, o2;
+          taylor_pair_at<R>(L, c, b, ph, &p1, &p2, o1, o2);
+          const C_t<R> po = base ? p2 : p1;
+          nz = !(rzero<R>(po.x) && rzero<R>(po.y));
+        }
+        __stcg(psi + b, p1);
+        __stcg(psi + (b ^ x), p2);
+        if (!nz || listed) return;
+        atomicOr(tb.cl.amask + (other >> 5), 1u << (other & 31u));
+        octet_set(mask, other);
+        if (own) {
+          const uint32_t at_own = atomicAdd(&s_n, 1u);
+          if (at_own < cap) {
+            list[at_own] = other;
+            return;
+          }
+        }
+        const uint32_t to = ((other * 0x9E3779B1u) >> 12) % G;
+        const uint32_t pos = atomicAdd(in_lens + 8u * to, 1u);
+        if (pos < seg) __stcg(inbox + (size_t)to * seg + pos, other);
+        else atomicOr(full_flag, 1u);   // no room: pairs are enumerated from the next step on
+      };
+      if (!full) {
+        for (;;) {
+          __syncwarp();
+          for (uint32_t q = lane; q < cnt; q += 32u) pair(wq[q]);
+          __syncwarp();
+          if (at >= n) break;
+          cnt = 0;   // entries that found no room in the queue, or are new rows
+          for (; at < n && cnt <= kListQueue - 32u; at += kSmemThreads) test(at + lane, at + lane < n);
+        }
+      } else {
+        const PairEnum& E = D.E;
+        const uint64_t count = (uint64_t)E.ncodes << E.log2cnt;
+        for (uint64_t q = rank * (uint64_t)kSmemThreads + threadIdx.x; q < count; q += (uint64_t)G * kSmemThreads) {
+          uint32_t ph;
+          const uint32_t b = enum_pair(E, (uint32_t)q, &ph), b2 = b ^ x;
+          const uint32_t w1 = __ldcg(mask + (b >> 8)), w2 = __ldcg(mask + (b2 >> 8));
+          const bool m1 = (w1 >> ((b >> 3) & 31u)) & 1u, m2 = (w2 >> ((b2 >> 3) & 31u)) & 1u;
+          if (!m1 && !m2) continue;
+          C_t<R> p1 = __ldcg(psi + b), p2 = __ldcg(psi + b2);
+          if constexpr (BACK) {
+            C_t<R> q1 = __ldcg(lam + b), q2 = __ldcg(lam + b2), o[4];
+            sum.add(adjoint_pair_at<R>(L, c, b, ph, &p1, &p2, &q1, &q2, o));
+            __stcg(lam + b, q1);
+            __stcg(lam + b2, q2);
+          } else {
+            C_t<R> o1, o2;
+            taylor_pair_at<R>(L, c, b, ph, &p1, &p2, o1, o2);
+          }
+          __stcg(psi + b, p1);
+          __stcg(psi + b2, p2);
+          if (!m1) octet_set(mask, b);
+          if (!m2) octet_set(mask, b2);
+        }
+        __syncwarp();
+      }
+    }
+    if constexpr (BACK) {
+      if (__any_sync(0xffffffffu, sum.any())) sum.warp();
+      if (lane == 0) s_sum[warp] = sum;
+    }
+    __syncthreads();
+    if (i + 1 < n_ops) {
+      if constexpr (CLUSTER) cluster_arrive();
+      else if (threadIdx.x == 0) red_release(bar);
+    }
+    n_list = min(s_n, cap);
+    if constexpr (BACK) {   // the step's partial, while the barrier completes
+      if (warp == kW - 1u) {
+        const double t = warp_sum(s_sum[lane].total());
+        if (lane == 0) dpart[(size_t)j * G + rank] = 2.0 * t;
+      }
+    }
+    if ((i + 1) % kListChunk == 0 && i + 1 < n_ops) {   // the next chunk's steps (their half of sd is free)
+      stage(i + 1);
+      __syncthreads();
+    }
+  }
 }
 
 // Whether one cluster of `blocks` blocks of `kernel` (kSmemThreads threads,
@@ -3116,8 +3568,10 @@ int launch_cluster(const void* kernel, int blocks, size_t bytes, void** args, cu
 // Whether the on-chip forward chain / backward sweep takes this problem.
 template <typename R>
 bool smem_chain_fits(const DeviceTables& d, int states) {
-  return d.t.pool_lut && onchip_mode(sizeof(R) == 4 ? GOCP_C64 : GOCP_C128) >= kOnchipBlock &&
-         ((uint64_t)states << d.t.n) * sizeof(C_t<R>) <= kSmemStateBytes;
+  return d.t.pool_lut && onchip_mode() >= kOnchipBlock &&
+         ((uint64_t)states << d.t.n) * sizeof(C_t<R>) <= kSmemStateBytes &&
+         !onchip_is("list") &&
+         (sizeof(R) == 4 || d.t.n <= kSmemC128Qubits || !onchip_is(nullptr));
 }
 
 // Opts the on-chip chain kernels into kSmemStateBytes of dynamic shared
@@ -3150,10 +3604,122 @@ int smem_chain_optin() {
                                  (int)(kSmemStateBytes + kSmemDescBytes));
       if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     }
+    for (const void* k : {(const void*)k_chain_list<R, false, false>, (const void*)k_chain_list<R, true, false>,
+                          (const void*)k_chain_list<R, false, true>, (const void*)k_chain_list<R, true, true>}) {
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)list_smem<R>());
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    }
     if (e != cudaSuccess) return cuda_status(e, "cudaFuncSetAttribute(on-chip chains)");
     done[device] = true;
   }
   return GOCP_OK;
+}
+
+// The most amplitudes that can be nonzero in a forward chain of n_ops
+// operators (back: in psi or H psi as well): the determinants of the reference
+// state's sector for a molecular problem, whose pool and H conserve the alpha
+// and beta electron counts (H only when no mapped term was dropped), else 2^n;
+// an operator at most doubles the number.
+uint64_t list_bound(const Problem& p, int n_ops, bool back) {
+  uint64_t b = 1ull << p.n_qubits;
+  if (p.n_elec >= 0 && !(back && p.terms_dropped)) {
+    const int no = p.n_qubits / 2, na = (p.n_elec + 1) / 2, nb = p.n_elec / 2;
+    auto binom = [](int n, int k) {
+      uint64_t c = 1;
+      for (int i = 1; i <= k; ++i) c = c * (uint64_t)(n - k + i) / (uint64_t)i;
+      return c;
+    };
+    if (na <= no) b = std::min(b, binom(no, na) * binom(no, nb));
+  }
+  if (!back && n_ops < 40) b = std::min<uint64_t>(b, 1ull << n_ops);
+  return b;
+}
+
+// Blocks that run a tracked chain (back: the adjoint sweep) as a list chain
+// (k_chain_list), 0: another form.  Measured, energy_grad of 40 operators, us
+// (one launch per step | list chain, 16 blocks of one cluster | every SM):
+//   complex64   14q 395 | 282 | 287    16q 400 | 333 | 352    18q 440 | 367 | 370    20q 518 | 459 | 415
+//   complex128  14q 556 | 468 | 497    16q 575 | 538 | 512    18q 745 | 698 | 541    20q 890 | 1159 | 682
+// so a short list takes the cluster, whose barrier is cheaper, and a longer one
+// every SM (complex128 sooner: its FP64 work on the touched pairs).  101
+// operators at 24 qubits: forward 5.3 -> 3.8 us a step, backward 6.1 -> 4.3.
+template <typename R>
+int list_chain_blocks(const Problem& p, int n_ops, bool back) {
+  const DeviceTables& d = *p.dev;
+  if (!d.t.pool_lut || !d.t.cl.list || !d.t.cl.sync) return 0;
+  const bool force = onchip_is("list");
+  if (!force && !onchip_is(nullptr)) return 0;
+  const uint64_t b = list_bound(p, n_ops, back);
+  // a state that may fill: the enumerated pairs, on every SM's own launches
+  if (!force && b == 1ull << p.n_qubits && b > kListMaxAny) return 0;
+  if (smem_chain_optin<R>() != GOCP_OK) return 0;
+  if (b <= (sizeof(R) == 4 ? kListClusterC64 : kListClusterC128) &&
+      cluster_fits(back ? (const void*)k_chain_list<R, true, true> : (const void*)k_chain_list<R, false, true>,
+                   kClusterMax, list_smem<R>()))
+    return kClusterMax;
+  return std::min(d.sm_count, kListMaxBlocks);
+}
+
+// Limit of a list chain's barrier wait: GOCP_CHAIN_WAIT_NS, default
+// kChainWaitNs; 0 gives up at once (a test drives that path).
+uint64_t chain_wait_ns() {
+  const char* e = std::getenv("GOCP_CHAIN_WAIT_NS");
+  if (!e || !*e) return kChainWaitNs;
+  const long long v = std::atoll(e);
+  return v < 0 ? kChainWaitNs : (uint64_t)v;
+}
+
+template <typename R>
+int launch_list_chain(Problem& p, int blocks, bool back, const int32_t* d_ops, int n_ops, void* psi, void* lam,
+                      double* d_dE, cudaStream_t st) {
+  DeviceTables& d = *p.dev;
+  DevTables tb = d.t;
+  const double* coefs = d.coefs;
+  int n = n_ops, slot = n_ops % 3;
+  C_t<R>* ps = (C_t<R>*)psi;
+  C_t<R>* ls = (C_t<R>*)lam;
+  uint32_t* mk = back ? d.t.octmask2 : d.t.octmask;
+  uint32_t ref = p.ref_index;
+  // inboxes: forward the chain list's own buffer, backward (where that holds
+  // the initial list) the amplitude list of H psi, which no chain needs
+  uint32_t* inbox = back ? d.chain_inbox : d.t.cl.list;
+  uint32_t seg = list_room(p.n_qubits) / (uint32_t)blocks;
+  double* dpart = d.dpart;
+  int32_t* err = d.err;
+  uint64_t wait = chain_wait_ns();
+  uint32_t cap = kListSmem;
+  if (const char* v = std::getenv("GOCP_LIST_SHARE")) cap = (uint32_t)std::min(std::max(std::atoi(v), 64), (int)kListSmem);
+  void* args[] = {&tb, &d_ops, &coefs, &n, &ps, &ls, &mk, &ref, &slot, &inbox, &seg, &dpart, &err, &cap, &wait};
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)blocks, 1, 1);
+  cfg.blockDim = dim3(kSmemThreads, 1, 1);
+  cfg.dynamicSmemBytes = list_smem<R>();
+  cfg.stream = st;
+  // the blocks wait for one another: one cluster, or a cooperative launch
+  cudaLaunchAttribute attr[1];
+  const void* k;
+  if (blocks == kClusterMax) {
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)blocks;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    k = back ? (const void*)k_chain_list<R, true, true> : (const void*)k_chain_list<R, false, true>;
+  } else {
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    k = back ? (const void*)k_chain_list<R, true, false> : (const void*)k_chain_list<R, false, false>;
+  }
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  ProfScope prof(back ? GOCP_KERNEL_ADJOINT : GOCP_KERNEL_TAYLOR, st, 1);
+  int rc = cuda_status(cudaLaunchKernelExC(&cfg, k, args), "list chain launch");
+  if (rc) return rc;
+  count_launches(1);
+  if (back) {
+    k_dtheta_reduce<<<n_ops, kThreads, 0, st>>>(dpart, blocks, d_dE);
+    count_launches(1);
+  }
+  return cuda_status(cudaGetLastError(), "list chain");
 }
 
 // ------------------------------------------------------------ launchers
@@ -3177,7 +3743,8 @@ int ensure_stage(Problem& p, int n_ops) {
       (rc = dalloc(d, &d.coefs, (size_t)cap * 6, bytes)) || (rc = dalloc(d, &d.dtheta, cap, bytes)))
     return rc;
   // per-block partials of the adjoint sweep (LUT pools): one row of blocks per op
-  if (d.t.pool_lut && (rc = dalloc(d, &d.dpart, (size_t)cap * adjoint_grid(d), bytes))) return rc;
+  if (d.t.pool_lut && (rc = dalloc(d, &d.dpart, (size_t)cap * std::max(adjoint_grid(d), d.sm_count), bytes)))
+    return rc;
   p.device_bytes += bytes;
   d.stage_cap = cap;
   return GOCP_OK;
@@ -3381,6 +3948,9 @@ static int launch_taylor_chain(Problem& p, const int32_t* d_ops, int n_ops, void
       return rc;
     }
   }
+  if (tracked && n_ops > 1)
+    if (const int lb = list_chain_blocks<R>(p, n_ops, false))   // over the nonzero amplitudes, in one launch
+      return launch_list_chain<R>(p, lb, false, d_ops, n_ops, psi, nullptr, nullptr, st);
   const int grid = d.t.pool_lut ? grid_for((uint64_t)d.t.penum_max, d.sm_count, kChainBlocksPerSm)
                                 : grid_for(1ull << (p.n_qubits - 1), d.sm_count, 8);
   uint32_t* mask = tracked && d.t.pool_lut ? d.t.octmask : nullptr;
@@ -3570,8 +4140,10 @@ static int launch_adjoint(Problem& p, const int32_t* d_ops, int n_ops, void* psi
       (rc = chain_list(p.precision, psi, lam, mask, p.n_qubits, d.t.cl, d.chain_counts, n_ops % 3,
                        (n_ops - 1) % 3, st)))
     return rc;
-  double* dpart = d.t.pool_lut ? d.dpart : nullptr;
   count_launches(1);   // k_residual (and k_octet_mask counts itself)
+  if (const int lb = mask && d.t.cl.list ? list_chain_blocks<R>(p, n_ops, true) : 0)
+    return launch_list_chain<R>(p, lb, true, d_ops, n_ops, psi, lam, d_dE, st);
+  double* dpart = d.t.pool_lut ? d.dpart : nullptr;
   DevTables tb = d.t;
   const double* coefs = d.coefs;
   int j = 0;
