@@ -27,6 +27,7 @@
 // are then undefined and gocp_device_errors reports the flag.
 #include <cuda.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdlib>
 
@@ -304,6 +305,8 @@ __global__ void __launch_bounds__(256) k_octet_mask(const C_t<R>* __restrict__ p
   }
 }
 
+constexpr int kTiledParts = 16;
+
 template <typename R>
 struct TiledArgs {
   const uint8_t* blob;
@@ -327,6 +330,12 @@ struct TiledArgs {
   const uint32_t* gate;
   uint32_t gate_max;
   uint64_t wait_ns;     // limit of a staging wait (stage_wait_ns)
+  // blocks per output tile: block part q takes the pieces [pbeg[q], pbeg[q + 1])
+  // and writes its sum to out (q = 0) or extra + (q - 1) 2^n; k_tiled_combine
+  // adds them up (K > 1)
+  int K;
+  C_t<R>* extra;
+  uint16_t pbeg[kTiledParts + 1];
 };
 
 template <typename R>
@@ -365,7 +374,8 @@ __host__ __device__ constexpr size_t tiled_smem() {
 #define GOCP_TILED_MINB_C64 1
 #endif
 
-template <typename R>
+// PARTS: several blocks per tile (TiledArgs::K > 1).
+template <typename R, bool PARTS>
 __global__ void __launch_bounds__(tiled_threads<R>(), sizeof(R) == 4 ? GOCP_TILED_MINB_C64 : 1)
     k_apply_h_tiled(const __grid_constant__ CUtensorMap tmap, const TiledArgs<R> a) {
   constexpr int LB = TiledBits<R>::LB;
@@ -393,8 +403,8 @@ __global__ void __launch_bounds__(tiled_threads<R>(), sizeof(R) == 4 ? GOCP_TILE
   // cost when zero octets are skipped), and the tile of each staged item is
   // passed to the consumers in s_tile; kNoTile ends the sweep.
   constexpr uint32_t kNoTile = 0xFFFFFFFFu;
-  const uint32_t ntiles = 1u << (a.n - LB);
-  __shared__ uint32_t s_tile[S], s_piece[S];
+  const uint32_t K = PARTS ? (uint32_t)a.K : 1u, nclaims = K << (a.n - LB);
+  __shared__ uint32_t s_tile[S], s_piece[S];   // claim (tile K + part) and piece of each stage
   // per-thread energy partials live in shared memory (touched once per tile)
   __shared__ double2 s_v[NT];
   s_v[threadIdx.x] = make_double2(0.0, 0.0);
@@ -411,7 +421,10 @@ __global__ void __launch_bounds__(tiled_threads<R>(), sizeof(R) == 4 ? GOCP_TILE
   // producer state, thread 0 only, kept in shared memory (not in every
   // thread's registers): items issued, piece and tile of the next, done
   __shared__ uint32_t s_next, s_pnext, s_tnext, s_done;
-  if (threadIdx.x == 0) s_next = s_pnext = s_tnext = s_done = 0u;
+  if (threadIdx.x == 0) {
+    s_next = s_tnext = s_done = 0u;
+    s_pnext = kNoTile;
+  }
   // thread 0: issue item s_next into stage s_next % S, whose previous item
   // every warp has released.  A piece whose source tile holds no nonzero
   // amplitude adds nothing and is passed over (never the last piece of a
@@ -421,24 +434,28 @@ __global__ void __launch_bounds__(tiled_threads<R>(), sizeof(R) == 4 ? GOCP_TILE
   auto issue_next = [&]() {
     const uint32_t st = s_next % S;
     const uint32_t fb = full_s + 8u * st;
-    uint32_t p = s_pnext, t = s_tnext;
+    uint32_t p = s_pnext, t = s_tnext, pend;
     for (;;) {
-      if (p == 0) t = atomicAdd(a.tile_counter, 1u);
-      if (t >= ntiles) {
+      if (p == kNoTile) {
+        t = atomicAdd(a.tile_counter, 1u);
+        p = PARTS ? a.pbeg[t % K] : 0u;
+      }
+      if (t >= nclaims) {
         s_tile[st] = kNoTile;
         asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(fb) : "memory");
         s_done = 1u;
         ++s_next;
         return;
       }
-      const uint32_t src = t ^ a.piece[p].xhi;
-      if (p + 1u == (uint32_t)a.n_pieces || !a.tile_flags || ((a.tile_flags[src >> 5] >> (src & 31u)) & 1u)) break;
+      const uint32_t src = (t / K) ^ a.piece[p].xhi;
+      pend = PARTS ? a.pbeg[t % K + 1u] : (uint32_t)a.n_pieces;
+      if (p + 1u == pend || !a.tile_flags || ((a.tile_flags[src >> 5] >> (src & 31u)) & 1u)) break;
       ++p;
     }
     s_tile[st] = t;
     s_piece[st] = p;
     const TiledPiece pc = a.piece[p];
-    const uint32_t src = t ^ pc.xhi;
+    const uint32_t src = (t / K) ^ pc.xhi;
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     mbar_expect_tx(fb, kTile + pc.bytes + kMask);
     const uint64_t keep = policy_evict_last();
@@ -449,7 +466,7 @@ __global__ void __launch_bounds__(tiled_threads<R>(), sizeof(R) == 4 ? GOCP_TILE
     bulk_copy(base_s + kMaskOff + st * kMask, reinterpret_cast<const uint8_t*>(a.mask) + (size_t)src * kMask, kMask,
               fb);
     ++s_next;
-    s_pnext = p + 1u == (uint32_t)a.n_pieces ? 0u : p + 1u;
+    s_pnext = p + 1u == pend ? kNoTile : p + 1u;
     s_tnext = t;
   };
   // Item j (j >= S) may reuse its stage once every warp has released item
@@ -485,6 +502,8 @@ __global__ void __launch_bounds__(tiled_threads<R>(), sizeof(R) == 4 ? GOCP_TILE
     }
     tile = s_tile[st];
     if (tile == kNoTile) break;   // the same item, so the same answer, for every warp
+    const uint32_t part = tile % K;
+    tile /= K;
     const int pc = (int)s_piece[st];
     {
       const uint32_t k0 = (tile << LB) + o * kAmpsH;
@@ -519,7 +538,15 @@ __global__ void __launch_bounds__(tiled_threads<R>(), sizeof(R) == 4 ? GOCP_TILE
           default: break;
         }
       }
-      if (pc == a.n_pieces - 1) {
+      if (PARTS && pc + 1 == (int)a.pbeg[part + 1u]) {
+        // this part's sum; the diagonal and the energy are k_tiled_combine's
+        C_t<R>* dst = (part ? a.extra + ((size_t)(part - 1u) << a.n) : a.out) + k0;
+#pragma unroll
+        for (int i = 0; i < kAmpsH; ++i) {
+          dst[i] = acc[i];
+          acc[i] = cmake<R>(0, 0);
+        }
+      } else if (!PARTS && pc == a.n_pieces - 1) {
         // the last piece has x >> LB = 0: tl is the own tile.  A zero own
         // octet adds nothing to the diagonal part or to the energy.
         C_t<R> res[kAmpsH];
@@ -582,8 +609,56 @@ __global__ void __launch_bounds__(tiled_threads<R>(), sizeof(R) == 4 ? GOCP_TILE
   }
   // (a normal exit consumed every issued item: nothing is in flight)
   const double v[2] = {s_v[threadIdx.x].x, s_v[threadIdx.x].y};
-  if (a.partials &&
+  if (a.partials && !PARTS &&
       block_grid_sum<2, NT>(v, a.partials, a.counter, gridDim.x, blockIdx.x, a.scal + 1, tot)) {
+    if (threadIdx.x == 0) a.scal[0] = a.identity + tot[1] / tot[0];
+  }
+}
+
+// out = the parts' sums (part 0 in out, then the K - 1 of extra, in order) plus
+// the diagonal group and the identity, with the energy partials; extra is
+// zeroed again (it is the scatter kernel's accumulator, zero between calls).
+// One octet per thread.
+template <typename R>
+__global__ void __launch_bounds__(256) k_tiled_combine(const C_t<R>* __restrict__ psi, const TiledArgs<R> a) {
+  if (a.gate && *a.gate <= a.gate_max) return;
+  __shared__ double tot[2];
+  double v[2] = {0.0, 0.0};
+  const uint32_t octets = 1u << (a.n - 3);
+  const R idr = (R)a.identity;
+  for (uint32_t o = blockIdx.x * 256u + threadIdx.x; o < octets; o += gridDim.x * 256u) {
+    const uint32_t k0 = o * kAmpsH;
+    C_t<R> acc[kAmpsH];
+#pragma unroll
+    for (int i = 0; i < kAmpsH; ++i) acc[i] = a.out[k0 + i];
+    for (int q = 1; q < a.K; ++q) {
+      C_t<R>* e = a.extra + ((size_t)(q - 1) << a.n) + k0;
+#pragma unroll
+      for (int i = 0; i < kAmpsH; ++i) {
+        acc[i] = cadd<R>(acc[i], e[i]);
+        e[i] = cmake<R>(0, 0);
+      }
+    }
+    if (octet_live(a.mask, o)) {
+      R dr[kAmpsH], dc[kAmpsH], di[kAmpsH], dd[kAmpsH];
+#pragma unroll
+      for (int i = 0; i < kAmpsH; ++i) dr[i] = dc[i] = di[i] = dd[i] = R(0);
+      sum_terms8<R>(a.dz, a.dw, 0, a.nd_mid, k0, dr, dc, true);
+      sum_terms8<R>(a.dz, a.dw, a.nd_mid, a.nd, k0, di, dd, false);
+#pragma unroll
+      for (int i = 0; i < kAmpsH; ++i) {
+        const C_t<R> p = psi[k0 + i];
+        const double pp = (double)p.x * p.x + (double)p.y * p.y;
+        v[0] += pp;
+        v[1] += (double)p.x * acc[i].x + (double)p.y * acc[i].y + ((double)dr[i] - (double)dc[i]) * pp;
+        const R d0 = dr[i] - dc[i] + idr;
+        acc[i] = cmake<R>(acc[i].x + d0 * p.x - di[i] * p.y, acc[i].y + d0 * p.y + di[i] * p.x);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < kAmpsH; ++i) a.out[k0 + i] = acc[i];
+  }
+  if (a.partials && block_grid_sum<2, 256>(v, a.partials, a.counter, gridDim.x, blockIdx.x, a.scal + 1, tot)) {
     if (threadIdx.x == 0) a.scal[0] = a.identity + tot[1] / tot[0];
   }
 }
@@ -616,8 +691,11 @@ int smem_optin(int device) {
   std::lock_guard<std::mutex> lk(mu);
   if (device >= (int)done.size()) done.resize(device + 1, false);
   if (!done[device]) {
-    cudaError_t e = cudaFuncSetAttribute(k_apply_h_tiled<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(k_apply_h_tiled<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)tiled_smem<R>());
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_apply_h_tiled<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)tiled_smem<R>());
     if (e != cudaSuccess) return cuda_status(e, "cudaFuncSetAttribute(k_apply_h_tiled)");
     done[device] = true;
   }
@@ -642,6 +720,18 @@ double sparse_frac() {
   if (!e || !*e) return 0.125;
   const double f = std::atof(e);
   return f < 0.0 ? 0.0 : (f > 0.25 ? 0.25 : f);
+}
+
+// First piece of part q of K: the pieces cut at equal shares of their bytes,
+// at least one piece to a part (K <= n_pieces).
+uint16_t tiled_cut(const DevTables& t, int q, int K) {
+  const std::vector<uint32_t>& off = *t.piece_off;
+  const int P = t.n_pieces;
+  if (q >= K) return (uint16_t)P;
+  const uint64_t want = (uint64_t)off[P] * (uint64_t)q / (uint64_t)K;
+  int p = (int)(std::lower_bound(off.begin(), off.end(), (uint32_t)want) - off.begin());
+  p = std::max(p, q);
+  return (uint16_t)std::min(p, P - (K - q));
 }
 
 template <typename R>
@@ -721,10 +811,40 @@ int launch_tiled(const DevTables& t, const LiveOctets& lv, int sm_count, const v
   a.err = err;
   a.wait_ns = stage_wait_ns();
   const uint64_t ntiles = 1ull << (t.n - LB);
+  // Fewer tiles than SMs: K blocks share a tile.  K (at most the room in
+  // extra, kTiledParts and the pieces allow) makes the rounds of equal parts
+  // over the SMs shortest; one more part has to shorten them by 4 % to pay for
+  // its pass.  Parts cut the pieces at equal shares of their bytes.  A dense
+  // state over 64 tiles, whose blocks left 88 of the 152 SMs idle: 4.44 -> 2.35
+  // ms (18 qubits complex128, K = 2), 247 -> 174 us (19-qubit all-pairs spin
+  // Hamiltonian, complex64, K = 3).
+  const uint64_t sms = (uint64_t)std::max(sm_count, 1);
+  int K = 1;
+  if (ntiles < sms && lv.gacc) {
+    const uint64_t room = 1ull + lv.gwords * sizeof(unsigned long long) / (sizeof(C_t<R>) << t.n);
+    const int kmax = (int)std::min<uint64_t>({(uint64_t)kTiledParts, room, (uint64_t)t.n_pieces});
+    double best = 1.0;
+    for (int k = 2; k <= kmax; ++k) {
+      const double r = (double)((ntiles * k + sms - 1) / sms) / k;
+      if (r < 0.96 * best) {
+        best = r;
+        K = k;
+      }
+    }
+  }
+  a.K = K;
+  a.extra = reinterpret_cast<C_t<R>*>(lv.gacc);
+  for (int q = 0; q <= K; ++q) a.pbeg[q] = tiled_cut(t, q, K);
   const int per_sm = sizeof(R) == 4 ? GOCP_TILED_MINB_C64 : 1;
-  const int grid = (int)std::min<uint64_t>(ntiles, (uint64_t)std::max(sm_count, 1) * per_sm);
-  k_apply_h_tiled<R><<<grid, tiled_threads<R>(), tiled_smem<R>(), st>>>(map, a);
+  const int grid = (int)std::min<uint64_t>(ntiles * K, sms * per_sm);
+  auto kern = K > 1 ? k_apply_h_tiled<R, true> : k_apply_h_tiled<R, false>;
+  kern<<<grid, tiled_threads<R>(), tiled_smem<R>(), st>>>(map, a);
   count_launches(1);
+  if (K > 1) {
+    const int cgrid = (int)std::min<uint64_t>(((1ull << (t.n - 3)) + 255) / 256, sms * 4);
+    k_tiled_combine<R><<<cgrid, 256, 0, st>>>(reinterpret_cast<const C_t<R>*>(psi), a);
+    count_launches(1);
+  }
   return cuda_status(cudaGetLastError(), "k_apply_h_tiled");
 }
 

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <vector>
 
 namespace gocp {
 
@@ -376,6 +377,7 @@ struct DevTables {
   int n_pieces = 0;
   const uint8_t* tblob = nullptr;
   const TiledPiece* tpiece = nullptr;
+  const std::vector<uint32_t>* piece_off = nullptr;   // host: byte offset of each piece, and the total
   SpTables sp;                  // the scatter kernel's form of the off-diagonal groups
   uint32_t* octmask = nullptr;
   uint32_t* tflags = nullptr;   // tiled form: one bit per tile (scratch)
@@ -616,6 +618,7 @@ struct LiveOctets {
   unsigned long long* gacc = nullptr;
   unsigned int* tdone = nullptr;
   uint32_t gtiles = 0;
+  size_t gwords = 0;   // words of gacc
 };
 
 // Lists the live octets of `mask` (2^(n-3) bits, n >= 8) into lv.list and

@@ -58,6 +58,7 @@ struct DeviceTables {
   DevTables t;
   int sm_count = 0;
   std::vector<void*> allocs;
+  std::vector<uint32_t> piece_off;   // DevTables::piece_off
   double* scratch = nullptr;
   size_t scratch_doubles = 0;
   unsigned int* counters = nullptr;  // kMaxChunks + 8
@@ -1993,8 +1994,7 @@ int build_scatter(int n, const std::vector<HLut<R>>& hl, const std::vector<uint3
           it.xo = 4u * (c.x & kLow);
           for (uint32_t q = 0; q < 4; ++q) {
             const uint32_t m = q == 3 ? c.z : q < c.nc ? c.m[q] : 0u, e = q == 3 ? c.ze : q < c.nc ? c.e[q] : 0u;
-            for (int b = 0; b < 32; ++b)
-              if ((m >> b) & 1u) bit[b][q] |= at;
+            for (uint32_t r = m; r; r &= r - 1u) bit[__builtin_ctz(r)][q] |= at;
             if (((uint32_t)parity32(c.x & kLow & m) ^ e) & 1u) c0[q] |= at;
             if (q < 3 && !(m & kLow)) fx[q] |= at;
           }
@@ -2509,16 +2509,21 @@ int build_tiled(int n, const std::vector<HLut<R>>& hl, const std::vector<uint32_
   // few output tiles (below 512: up to 21 qubits): global accumulators for
   // the scatter kernel's blocks that share a tile, zero between calls
   if (ntiles < 512) {
-    const size_t words = ntiles * (size_t)kSpTile * 2u;
+    // (8 MiB at least: the staged kernel's parts of a small state go there too)
+    const size_t words = std::max(ntiles * (size_t)kSpTile * 2u, (size_t)1 << 20);
     if ((rc = dalloc(d, &d.live.gacc, words, bytes)) || (rc = dalloc(d, &d.live.tdone, ntiles, bytes))) return rc;
     if ((rc = cuda_status(cudaMemset(d.live.gacc, 0, words * sizeof(unsigned long long)), "zero gacc")) ||
         (rc = cuda_status(cudaMemset(d.live.tdone, 0, ntiles * sizeof(unsigned int)), "zero tdone")))
       return rc;
     d.live.gtiles = (uint32_t)ntiles;
+    d.live.gwords = words;
   }
   d.t.tblob = dblob;
   d.t.tpiece = dpiece;
   d.t.n_pieces = (int)pieces.size();
+  for (const TiledPiece& pc : pieces) d.piece_off.push_back(pc.off);
+  d.piece_off.push_back((uint32_t)blob.size());
+  d.t.piece_off = &d.piece_off;
   return GOCP_OK;
 }
 
