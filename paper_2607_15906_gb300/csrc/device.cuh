@@ -53,6 +53,33 @@ __device__ __forceinline__ void chain_step_begin() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// Barrier between the blocks of a cooperative launch: a count in global memory
+// (zero at the launch).  grid_arrive by one thread after a block barrier, so
+// that the block's writes come before it; grid_wait by one thread before one,
+// false (recorded in err) when the count has not reached `want` after wait_ns
+// (0: at once).
+constexpr int32_t kErrChainTimeout = 4;
+__device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void grid_arrive(uint32_t* bar) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+}
+__device__ __forceinline__ bool grid_wait(const uint32_t* bar, uint32_t want, uint64_t wait_ns, int32_t* err) {
+  uint64_t t0, t1;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+  for (uint32_t spin = 1; wait_ns != 0; ++spin) {
+    if (ld_acquire(bar) >= want) return true;
+    if ((spin & 1023u) != 0u) continue;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
+    if (t1 - t0 > wait_ns) break;
+  }
+  atomicOr(err, kErrChainTimeout);
+  return false;
+}
+
 // An x-group (or generator) in LUT form, see LutForm:
 //   D(b) = (-1)^popc(b & z0) * lut[phi(b)],  phi(b) = sum_i (popc(b & v_i) & 1) << i,
 // with real weights only.  fx holds phi(x) (bits 0..2) and popc(x & z0) & 1
@@ -698,6 +725,10 @@ double* scratch_ptr(Problem& p, size_t* doubles);
 unsigned int* counters_ptr(Problem& p);
 int pool_finish(Problem& p, const double* part, int nbx, double* d_grads, cudaStream_t st);
 int ensure_stage(Problem& p, int n_ops);
+double* dpart_ptr(Problem& p);          // stage capacity x at least the SM count
+bool chain_forms_default();             // GOCP_ONCHIP_CHAINS is unset
+uint64_t chain_wait_ns();               // limit of a wait between the blocks of a chain
+int dtheta_reduce(Problem& p, int blocks, int n_ops, double* d_dE, cudaStream_t st);
 double* scalars_ptr(Problem& p);
 int32_t* err_ptr(Problem& p);
 int dev_norm(Problem& p, const void* psi, cudaStream_t st);

@@ -3161,7 +3161,6 @@ constexpr uint32_t kListSmem = 24576;    // entries of a block's share in shared
 constexpr uint32_t kListOwn = 64;        // share from which a block keeps its new entries
 constexpr uint32_t kListQueue = 512;     // queued entries per warp
 constexpr int kListChunk = 32;           // steps staged at a time
-constexpr int32_t kErrChainTimeout = 4;
 constexpr uint64_t kChainWaitNs = 2000000000ull;   // limit of a barrier wait: 2 s
 
 template <typename R>
@@ -3208,16 +3207,6 @@ template <> struct StepSum<double> { using T = DoubleSum; };
 
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
-__device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
-  uint32_t v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-
-__device__ __forceinline__ void red_release(uint32_t* p) {
-  asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p) : "memory");
-}
-
 // BACK false: psi <- the chain applied to psi, starting from the list {ref}
 // (the reference state dev_setup wrote).  BACK true: the adjoint sweep over
 // psi and lam, from the list chain_list wrote (its length in ring slot
@@ -3339,24 +3328,7 @@ k_chain_list(DevTables tb, const int32_t* ops, const double* coefs, int n_ops, C
       // same round trip, the first 32 entries it may have gained
       if constexpr (CLUSTER) cluster_wait();
       if (warp == 0) {
-        if (!CLUSTER && lane == 0) {
-          const uint32_t want = (uint32_t)i * G;
-          if (wait_ns == 0 || ld_acquire(bar) < want) {
-            uint64_t t0, t1;
-            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
-            for (uint32_t spin = 0;; ++spin) {
-              if (wait_ns != 0 && ld_acquire(bar) >= want) break;
-              if (wait_ns == 0 || (spin & 1023u) == 1023u) {
-                asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
-                if (wait_ns == 0 || t1 - t0 > wait_ns) {
-                  atomicOr(err, kErrChainTimeout);
-                  s_abort = 1;
-                  break;
-                }
-              }
-            }
-          }
-        }
+        if (!CLUSTER && lane == 0 && !grid_wait(bar, (uint32_t)i * G, wait_ns, err)) s_abort = 1;
         __syncwarp();
         const uint32_t got = min(__ldcg(in_lens + 8u * rank), seg), over = __ldcg(full_flag);
         const uint32_t q = in_len + lane, early = q < seg ? __ldcg(mine_in + q) : 0u;
@@ -3490,7 +3462,7 @@ k_chain_list(DevTables tb, const int32_t* ops, const double* coefs, int n_ops, C
     __syncthreads();
     if (i + 1 < n_ops) {
       if constexpr (CLUSTER) cluster_arrive();
-      else if (threadIdx.x == 0) red_release(bar);
+      else if (threadIdx.x == 0) grid_arrive(bar);
     }
     n_list = min(s_n, cap);
     if constexpr (BACK) {   // the step's partial, while the barrier completes
@@ -3674,6 +3646,15 @@ uint64_t chain_wait_ns() {
   const long long v = std::atoll(e);
   return v < 0 ? kChainWaitNs : (uint64_t)v;
 }
+bool chain_forms_default() { return onchip_is(nullptr); }
+double* dpart_ptr(Problem& p) { return p.dev->dpart; }
+
+// d_dE[j] = the sum of dpart[j blocks .. (j + 1) blocks), in order.
+int dtheta_reduce(Problem& p, int blocks, int n_ops, double* d_dE, cudaStream_t st) {
+  k_dtheta_reduce<<<n_ops, kThreads, 0, st>>>(p.dev->dpart, blocks, d_dE);
+  count_launches(1);
+  return cuda_status(cudaGetLastError(), "k_dtheta_reduce");
+}
 
 template <typename R>
 int launch_list_chain(Problem& p, int blocks, bool back, const int32_t* d_ops, int n_ops, void* psi, void* lam,
@@ -3720,11 +3701,7 @@ int launch_list_chain(Problem& p, int blocks, bool back, const int32_t* d_ops, i
   int rc = cuda_status(cudaLaunchKernelExC(&cfg, k, args), "list chain launch");
   if (rc) return rc;
   count_launches(1);
-  if (back) {
-    k_dtheta_reduce<<<n_ops, kThreads, 0, st>>>(dpart, blocks, d_dE);
-    count_launches(1);
-  }
-  return cuda_status(cudaGetLastError(), "list chain");
+  return back ? dtheta_reduce(p, blocks, n_ops, d_dE, st) : GOCP_OK;
 }
 
 // ------------------------------------------------------------ launchers
@@ -4163,10 +4140,7 @@ static int launch_adjoint(Problem& p, const int32_t* d_ops, int n_ops, void* psi
   ProfScope ps(GOCP_KERNEL_ADJOINT, st, n_ops + (dpart ? 1 : 0));
   if ((rc = launch_chain(p, (const void*)k_adjoint<R>, grid, kThreads, n_ops, true, args, sizes, 12, 3, st)))
     return rc;
-  if (dpart) {
-    k_dtheta_reduce<<<n_ops, kThreads, 0, st>>>(dpart, grid, d_dE);
-    count_launches(1);
-  }
+  if (dpart && (rc = dtheta_reduce(p, grid, n_ops, d_dE, st))) return rc;
   return cuda_status(cudaGetLastError(), "k_adjoint");
 }
 

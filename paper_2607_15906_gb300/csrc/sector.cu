@@ -71,7 +71,8 @@ __device__ __forceinline__ void kahan(R& s, R& c, R v) {
 // psi = row ref; block 0 also writes coefs[6j + m] = theta_j^m / m!.
 template <typename R>
 __global__ void __launch_bounds__(kSecThreads)
-k_sec_setup(C_t<R>* psi, int32_t D, int32_t ref, const double* theta, int n_ops, double* coefs) {
+k_sec_setup(C_t<R>* psi, int32_t D, int32_t ref, const double* theta, int n_ops, double* coefs, uint32_t* sync) {
+  if (sync && blockIdx.x == 0 && threadIdx.x == 0) sync[kSyncBar] = 0u;   // for the chain that follows
   if (psi)
     for (int32_t r = blockIdx.x * kSecThreads + threadIdx.x; r < D; r += gridDim.x * kSecThreads)
       psi[r] = cmake<R>(r == ref ? R(1) : R(0), R(0));
@@ -84,6 +85,60 @@ k_sec_setup(C_t<R>* psi, int32_t D, int32_t ref, const double* theta, int n_ops,
         coefs[6 * j + m] = c;
       }
     }
+}
+
+// (v1, v2) <- T (v1, v2) on a pair with couplings d1, d2.
+template <typename R>
+__device__ __forceinline__ void sec_taylor_pair(R d1, R d2, const R (&c)[6], C_t<R>& v1, C_t<R>& v2) {
+  if constexpr (sizeof(R) == 8) {
+    // complex128: the same polynomial through A^2 = mu I on the pair (see
+    // taylor_pair_at in kernels.cu)
+    const R mu = d1 * d2, mu2 = mu * mu;
+    const R cc = c[0] + c[2] * mu + c[4] * mu2;
+    const R sc = c[1] + c[3] * mu + c[5] * mu2;
+    const R sd1 = sc * d1, sd2 = sc * d2;
+    const C_t<R> o1 = cmake<R>(cc * v1.x + sd1 * v2.x, cc * v1.y + sd1 * v2.y);
+    v2 = cmake<R>(cc * v2.x + sd2 * v1.x, cc * v2.y + sd2 * v1.y);
+    v1 = o1;
+    return;
+  }
+  C_t<R> s1 = v1, s2 = v2, e1 = cmake<R>(0, 0), e2 = cmake<R>(0, 0);
+#pragma unroll
+  for (int m = 1; m <= 5; ++m) {
+    const C_t<R> n1 = cscale<R>(v2, d1), n2 = cscale<R>(v1, d2);   // (A v)[k] = D(k) v[k ^ x]
+    v1 = n1;
+    v2 = n2;
+    kahan<R>(s1.x, e1.x, v1.x * c[m]);
+    kahan<R>(s1.y, e1.y, v1.y * c[m]);
+    kahan<R>(s2.x, e2.x, v2.x * c[m]);
+    kahan<R>(s2.y, e2.y, v2.y * c[m]);
+  }
+  v1 = csub<R>(s1, e1);
+  v2 = csub<R>(s2, e2);
+}
+
+// The backward step on a pair: u <- T^-1 u exactly, l <- T^dagger l; returns
+// 2 Re<l|T' u>.
+template <typename R>
+__device__ __forceinline__ R sec_adjoint_pair(R d1, R d2, const R (&c)[6], C_t<R>& u1, C_t<R>& u2, C_t<R>& l1v,
+                                              C_t<R>& l2v) {
+  const R mu = d1 * d2, mu2 = mu * mu;
+  const R cc = c[0] + c[2] * mu + c[4] * mu2;
+  const R sc = c[1] + c[3] * mu + c[5] * mu2;
+  const R cd = c[1] * mu + c[3] * mu2;
+  const R inv = R(1) / (cc * cc - sc * sc * mu);
+  const R sd1 = sc * d1, sd2 = sc * d2;
+  const C_t<R> q1 = cscale<R>(csub<R>(cscale<R>(u1, cc), cscale<R>(u2, sd1)), inv);
+  const C_t<R> q2 = cscale<R>(csub<R>(cscale<R>(u2, cc), cscale<R>(u1, sd2)), inv);
+  const C_t<R> t1 = cadd<R>(cscale<R>(q1, cd), cscale<R>(q2, cc * d1));
+  const C_t<R> t2 = cadd<R>(cscale<R>(q2, cd), cscale<R>(q1, cc * d2));
+  const R v = R(2) * (l1v.x * t1.x + l1v.y * t1.y + l2v.x * t2.x + l2v.y * t2.y);
+  u1 = q1;
+  u2 = q2;
+  const C_t<R> m1 = cadd<R>(cscale<R>(l1v, cc), cscale<R>(l2v, sd2));
+  l2v = cadd<R>(cscale<R>(l1v, sd1), cscale<R>(l2v, cc));
+  l1v = m1;
+  return v;
 }
 
 // One Taylor step (Eq. 5, 6) of generator ops[j] in LUT form over its pair
@@ -111,30 +166,9 @@ k_sec_taylor(SecDev s, DevTables tb, const uint2* pairs, const int64_t* off, con
     const uint32_t sg = __popc(k & L.z0) & 1u;
     const R d1 = sg ? -l1 : l1, d2 = (sg ^ sgx) ? -l2 : l2;
     C_t<R> v1 = psi[pr.x], v2 = psi[pr.y];
-    if constexpr (sizeof(R) == 8) {
-      // complex128: the same polynomial through A^2 = mu I on the pair (see
-      // taylor_pair_at in kernels.cu)
-      const R mu = d1 * d2, mu2 = mu * mu;
-      const R cc = c[0] + c[2] * mu + c[4] * mu2;
-      const R sc = c[1] + c[3] * mu + c[5] * mu2;
-      const R sd1 = sc * d1, sd2 = sc * d2;
-      psi[pr.x] = cmake<R>(cc * v1.x + sd1 * v2.x, cc * v1.y + sd1 * v2.y);
-      psi[pr.y] = cmake<R>(cc * v2.x + sd2 * v1.x, cc * v2.y + sd2 * v1.y);
-      continue;
-    }
-    C_t<R> s1 = v1, s2 = v2, e1 = cmake<R>(0, 0), e2 = cmake<R>(0, 0);
-#pragma unroll
-    for (int m = 1; m <= 5; ++m) {
-      const C_t<R> n1 = cscale<R>(v2, d1), n2 = cscale<R>(v1, d2);   // (A v)[k] = D(k) v[k ^ x]
-      v1 = n1;
-      v2 = n2;
-      kahan<R>(s1.x, e1.x, v1.x * c[m]);
-      kahan<R>(s1.y, e1.y, v1.y * c[m]);
-      kahan<R>(s2.x, e2.x, v2.x * c[m]);
-      kahan<R>(s2.y, e2.y, v2.y * c[m]);
-    }
-    psi[pr.x] = csub<R>(s1, e1);
-    psi[pr.y] = csub<R>(s2, e2);
+    sec_taylor_pair<R>(d1, d2, c, v1, v2);
+    psi[pr.x] = v1;
+    psi[pr.y] = v2;
   }
 }
 
@@ -318,7 +352,8 @@ k_sec_spmv(int32_t D, const int64_t* __restrict__ ptr, const uint32_t* __restric
 // lambda = (H psi - E psi) / <psi|psi> in place (E, <psi|psi> = scal[0..1]).
 template <typename R>
 __global__ void __launch_bounds__(kSecThreads)
-k_sec_residual(const C_t<R>* psi, C_t<R>* lam, int32_t D, const double* scal) {
+k_sec_residual(const C_t<R>* psi, C_t<R>* lam, int32_t D, const double* scal, uint32_t* sync) {
+  if (sync && blockIdx.x == 0 && threadIdx.x == 0) sync[kSyncBar] = 0u;   // for the sweep that follows
   const R er = (R)scal[0], ir = (R)(1.0 / scal[1]);
   for (int32_t r = blockIdx.x * kSecThreads + threadIdx.x; r < D; r += gridDim.x * kSecThreads) {
     const C_t<R> h = lam[r], p = psi[r];
@@ -403,26 +438,128 @@ k_sec_adjoint(SecDev s, DevTables tb, const uint2* pairs, const int64_t* off, co
     const R l1 = L.lut[ph], l2 = L.lut[ph ^ phx];
     const uint32_t sg = __popc(k & L.z0) & 1u;
     const R d1 = sg ? -l1 : l1, d2 = (sg ^ sgx) ? -l2 : l2;
-    const R mu = d1 * d2, mu2 = mu * mu;
-    const R cc = c[0] + c[2] * mu + c[4] * mu2;
-    const R sc = c[1] + c[3] * mu + c[5] * mu2;
-    const R cd = c[1] * mu + c[3] * mu2;
-    const R inv = R(1) / (cc * cc - sc * sc * mu);
-    const R sd1 = sc * d1, sd2 = sc * d2;
-    const C_t<R> u1 = psi[pr.x], u2 = psi[pr.y];
-    const C_t<R> q1 = cscale<R>(csub<R>(cscale<R>(u1, cc), cscale<R>(u2, sd1)), inv);
-    const C_t<R> q2 = cscale<R>(csub<R>(cscale<R>(u2, cc), cscale<R>(u1, sd2)), inv);
-    const C_t<R> t1 = cadd<R>(cscale<R>(q1, cd), cscale<R>(q2, cc * d1));
-    const C_t<R> t2 = cadd<R>(cscale<R>(q2, cd), cscale<R>(q1, cc * d2));
-    const C_t<R> l1v = lam[pr.x], l2v = lam[pr.y];
-    kahan<R>(acc, cmp, R(2) * (l1v.x * t1.x + l1v.y * t1.y + l2v.x * t2.x + l2v.y * t2.y));
-    psi[pr.x] = q1;
-    psi[pr.y] = q2;
-    lam[pr.x] = cadd<R>(cscale<R>(l1v, cc), cscale<R>(l2v, sd2));
-    lam[pr.y] = cadd<R>(cscale<R>(l1v, sd1), cscale<R>(l2v, cc));
+    C_t<R> u1 = psi[pr.x], u2 = psi[pr.y], l1v = lam[pr.x], l2v = lam[pr.y];
+    kahan<R>(acc, cmp, sec_adjoint_pair<R>(d1, d2, c, u1, u2, l1v, l2v));
+    psi[pr.x] = u1;
+    psi[pr.y] = u2;
+    lam[pr.x] = l1v;
+    lam[pr.y] = l2v;
   }
   const double v[1] = {(double)warp_total<R>(acc - cmp)};
   block_grid_sum<1, kSecThreads, true>(v, partials, counter, gridDim.x, blockIdx.x, dtheta + j, tot);
+}
+
+// The whole chain (BACK: the whole backward sweep) in one cooperative launch,
+// the blocks waiting for one another between steps.  The pair lists do not
+// depend on the state, so a thread has its pair of the next step, and the
+// couplings on it, before the barrier completes; a step is then one read of
+// the amplitudes, the arithmetic, one write and the barrier.  Warps of pairs go
+// round the blocks, so that a short list keeps every SM's FP64 pipe and load
+// unit busy for the shortest time.  dpart[j G + block] = the block's part of
+// dE_j.  sync: the barrier's count, zero at the start.
+constexpr int kSecChainThreads = 1024;
+constexpr int kSecChunkSteps = 32;   // steps staged at a time
+template <typename R>
+struct SecStep {
+  LutDev<R> L;
+  R c[6];
+  uint32_t np;
+  int32_t valid;   // 0: the operator index was out of range (the step is the identity)
+  int64_t q0;
+};
+
+template <typename R, bool BACK>
+__global__ void __launch_bounds__(kSecChainThreads, 1)
+k_sec_chain(SecDev s, DevTables tb, const uint2* __restrict__ pairs, const int64_t* __restrict__ off,
+            const int32_t* ops, const double* coefs, int n_ops, C_t<R>* psi, C_t<R>* lam, uint32_t* sync,
+            double* dpart, int32_t* err, uint64_t wait_ns) {
+  __shared__ SecStep<R> sd[2 * kSecChunkSteps];
+  __shared__ double s_sum[kSecChainThreads / 32];
+  __shared__ int s_abort;
+  constexpr uint32_t kW = kSecChainThreads / 32;
+  const uint32_t G = gridDim.x, rank = blockIdx.x, lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  uint32_t* bar = sync + kSyncBar;
+  auto stage = [&](int i) {   // steps i .. i + kSecChunkSteps - 1 into their half of sd
+    for (int q = (int)warp; q < min(n_ops - i, kSecChunkSteps); q += (int)kW) {
+      const int jq = BACK ? n_ops - 1 - (i + q) : i + q, op = ops[jq];
+      SecStep<R>& D = sd[(i + q) % (2 * kSecChunkSteps)];
+      const bool ok = op >= 0 && op < tb.M;
+      if (lane == 0) {
+        D.valid = ok ? 1 : 0;
+        D.q0 = ok ? off[op] : 0;
+        D.np = ok ? (uint32_t)(off[op + 1] - off[op]) : 0u;
+        if (!ok && rank == 0) atomicOr(err, 1);
+        if (ok) D.L = ((const LutDev<R>*)tb.plut)[op];
+      }
+      if (ok && lane < 6) D.c[lane] = (R)coefs[6 * jq + lane];
+    }
+  };
+  if (threadIdx.x == 0) s_abort = 0;
+  stage(0);
+  __syncthreads();
+  for (int i = 0; i < n_ops; ++i) {
+    const int j = BACK ? n_ops - 1 - i : i;
+    const SecStep<R>& D = sd[i % (2 * kSecChunkSteps)];
+    const LutDev<R>& L = D.L;
+    uint2 pr = make_uint2(0u, 0u);
+    R d1 = R(0), d2 = R(0);
+    auto fetch = [&](uint32_t e) {   // pair e of the step and its couplings
+      pr = __ldg(pairs + D.q0 + e);
+      const uint32_t k = __ldg(s.kq + pr.x), ph = lut_phi(L, k);
+      const R l1 = L.lut[ph], l2 = L.lut[ph ^ (L.fx & 7u)];
+      const uint32_t sg = __popc(k & L.z0) & 1u;
+      d1 = sg ? -l1 : l1;
+      d2 = (sg ^ ((L.fx >> 3) & 1u)) ? -l2 : l2;
+    };
+    uint32_t e = (warp * G + rank) * 32u + lane;
+    if (e < D.np) fetch(e);
+    R c[6];
+#pragma unroll
+    for (int m = 0; m < 6; ++m) c[m] = D.c[m];
+    if (i > 0 && G > 1u) {
+      if (threadIdx.x == 0 && !grid_wait(bar, (uint32_t)i * G, wait_ns, err)) s_abort = 1;
+      __syncthreads();
+      if (s_abort) return;
+    }
+    // a thread's part of dE_j is compensated in R; warps sum in R, the block in
+    // FP64 (a slow pipe on this part)
+    R acc = R(0), cmp = R(0);
+    while (e < D.np) {
+      C_t<R> v1 = __ldcg(psi + pr.x), v2 = __ldcg(psi + pr.y);
+      if constexpr (BACK) {
+        C_t<R> l1 = __ldcg(lam + pr.x), l2 = __ldcg(lam + pr.y);
+        kahan<R>(acc, cmp, sec_adjoint_pair<R>(d1, d2, c, v1, v2, l1, l2));
+        __stcg(lam + pr.x, l1);
+        __stcg(lam + pr.y, l2);
+      } else {
+        sec_taylor_pair<R>(d1, d2, c, v1, v2);
+      }
+      __stcg(psi + pr.x, v1);
+      __stcg(psi + pr.y, v2);
+      e += G * kSecChainThreads;
+      if (e < D.np) fetch(e);
+    }
+    __syncwarp();
+    if constexpr (BACK) {
+      R v = acc - cmp;
+      if (__any_sync(0xffffffffu, !rzero<R>(v))) v = warp_total<R>(v);
+      if (lane == 0) s_sum[warp] = (double)v;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && i + 1 < n_ops && G > 1u) grid_arrive(bar);
+    if constexpr (BACK) {   // the step's partial, while the barrier completes
+      if (warp == kW - 1u) {
+        const double t = warp_sum(s_sum[lane]);
+        if (lane == 0) dpart[(size_t)j * G + rank] = t;
+      }
+    }
+    if ((i + 1) % kSecChunkSteps == 0 && i + 1 < n_ops) {
+      stage(i + 1);
+      __syncthreads();
+    } else if (G == 1u && BACK) {
+      __syncthreads();   // s_sum is read before the next step writes it (with more blocks, the barrier's wait)
+    }
+  }
 }
 
 template <typename R>
@@ -544,8 +681,52 @@ int pair_grid(Problem& p, int per_sm) {
   return (int)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)sm_of(p) * per_sm));
 }
 
+// Blocks of a cooperative sector chain, 0: a launch per step (asked for by
+// GOCP_ONCHIP_CHAINS = "off", or no barrier word: below 8 qubits).  256 pairs of
+// the longest list per block, at most every SM: with fewer the barrier costs
+// more than the shares save.
+int sec_chain_blocks(Problem& p, int n_ops) {
+  if (n_ops < 2 || !dev_tables(p).cl.sync || !chain_forms_default()) return 0;
+  return (int)std::max<int64_t>(1, std::min<int64_t>(sm_of(p), (p.sec->max_pairs + 255) / 256));
+}
+
+template <typename R>
+int launch_sec_chain(Problem& p, int blocks, bool back, const int32_t* d_ops, int n_ops, void* psi, void* lam,
+                     double* d_dE, cudaStream_t st) {
+  SecDev sd = p.sec->s;
+  DevTables tb = dev_tables(p);
+  const uint2* pairs = p.sec->pairs;
+  const int64_t* off = p.sec->off;
+  const double* coefs = coefs_ptr(p);
+  int n = n_ops;
+  C_t<R>* ps = (C_t<R>*)psi;
+  C_t<R>* ls = (C_t<R>*)lam;
+  uint32_t* sync = tb.cl.sync;
+  double* dpart = dpart_ptr(p);
+  int32_t* err = err_ptr(p);
+  uint64_t wait = chain_wait_ns();
+  void* args[] = {&sd, &tb, &pairs, &off, &d_ops, &coefs, &n, &ps, &ls, &sync, &dpart, &err, &wait};
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)blocks, 1, 1);
+  cfg.blockDim = dim3(kSecChainThreads, 1, 1);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;   // every block resident: they wait for one another
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  ProfScope prof(back ? GOCP_KERNEL_ADJOINT : GOCP_KERNEL_TAYLOR, st, 1);
+  const void* k = back ? (const void*)k_sec_chain<R, true> : (const void*)k_sec_chain<R, false>;
+  const int rc = cuda_status(cudaLaunchKernelExC(&cfg, k, args), "sector chain launch");
+  if (rc) return rc;
+  count_launches(1);
+  return back ? dtheta_reduce(p, blocks, n_ops, d_dE, st) : GOCP_OK;
+}
+
 template <typename R>
 int sec_taylor_t(Problem& p, const int32_t* d_ops, int n_ops, void* psi, cudaStream_t st) {
+  if (const int b = sec_chain_blocks(p, n_ops))
+    return launch_sec_chain<R>(p, b, false, d_ops, n_ops, psi, nullptr, nullptr, st);
   const int grid = pair_grid(p, 8);
   SecDev sd = p.sec->s;
   DevTables tb = dev_tables(p);
@@ -595,8 +776,10 @@ int sec_adjoint_t(Problem& p, const int32_t* d_ops, int n_ops, void* psi, void* 
   size_t nd = 0;
   double* scratch = scratch_ptr(p, &nd);
   k_sec_residual<R><<<grid_rows(D, sm_of(p), 8), kSecThreads, 0, st>>>((const C_t<R>*)psi, (C_t<R>*)lam, D,
-                                                                       scalars_ptr(p));
+                                                                       scalars_ptr(p), dev_tables(p).cl.sync);
   count_launches(1);   // k_sec_residual
+  if (const int b = sec_chain_blocks(p, n_ops))
+    return launch_sec_chain<R>(p, b, true, d_ops, n_ops, psi, lam, d_dE, st);
   const int grid = std::min<int>(pair_grid(p, 2), (int)nd);
   SecDev sd = p.sec->s;
   DevTables tb = dev_tables(p);
@@ -824,10 +1007,10 @@ int sec_setup(Problem& p, void* psi, const double* d_theta, int n_ops, void* str
   const int grid = psi ? grid_rows(p.sector_dim, sm_of(p), 8) : 1;
   if (p.precision == GOCP_C64)
     k_sec_setup<float><<<grid, kSecThreads, 0, st>>>((float2*)psi, p.sec->s.D, p.sec->ref_row, d_theta, n_ops,
-                                                     coefs_ptr(p));
+                                                     coefs_ptr(p), dev_tables(p).cl.sync);
   else
     k_sec_setup<double><<<grid, kSecThreads, 0, st>>>((double2*)psi, p.sec->s.D, p.sec->ref_row, d_theta, n_ops,
-                                                      coefs_ptr(p));
+                                                      coefs_ptr(p), dev_tables(p).cl.sync);
   count_launches(1);
   return cuda_status(cudaGetLastError(), "k_sec_setup");
 }

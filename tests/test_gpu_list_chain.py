@@ -127,3 +127,34 @@ def test_list_chain_wait_runs_out(monkeypatch):
     monkeypatch.delenv("GOCP_CHAIN_WAIT_NS")
     p.prepare_state(ops, th, got)
     assert p.device_errors() == 0 and torch.equal(want, got)
+
+
+@pytest.mark.parametrize("prec", ["c128", "c64"])
+@pytest.mark.parametrize("n_orb,n_elec", [(4, 3), (6, 6), (9, 8)])
+def test_sector_chain_equals_a_launch_per_step(prec, n_orb, n_elec, monkeypatch):
+    """The sector layout's chains in one launch (one block, and several waiting
+    for one another; 70 operators: more than one staged chunk) against a launch
+    per step: the state bit for bit, dE/dtheta to rounding, twice the same; an
+    operator out of range is flagged and acts as the identity."""
+    ints = molecular_integrals(n_orb, seed=2, decay=True)
+    p = gb.Problem.build(ints, n_elec, precision=prec, device=0, sector=True)
+    ops, th = draw_ansatz(p.pool_size, 70, seed=4, theta_sigma=0.3)
+    out = {}
+    for mode in ("off", None):
+        if mode:
+            monkeypatch.setenv("GOCP_ONCHIP_CHAINS", mode)
+        else:
+            monkeypatch.delenv("GOCP_ONCHIP_CHAINS")
+        d = p.new_states(1)[0]
+        p.prepare_state(ops, th, d)
+        out[mode] = (d, *p.energy_grad(ops, th))
+    assert p.device_errors() == 0
+    assert torch.equal(out["off"][0], out[None][0]) and out["off"][1] == out[None][1]
+    assert np.max(np.abs(out["off"][2] - out[None][2])) <= TOL[prec][2] * max(1.0, np.max(np.abs(out["off"][2])))
+    e, de = p.energy_grad(ops, th)
+    assert e == out[None][1] and np.array_equal(de, out[None][2])
+    good, bad = p.new_states(2)
+    p.prepare_state(np.delete(ops, 40), np.delete(th, 40), good)
+    ops[40] = p.pool_size
+    p.prepare_state(torch.from_numpy(ops).cuda(), torch.from_numpy(th).cuda(), bad)
+    assert p.device_errors() == 1 and torch.equal(good, bad)
