@@ -548,8 +548,18 @@ constexpr uint32_t kSpMaxSmem = 224u << 10;   // of the 227 KB a block can have
 // The part of head q's words that tile t gives.
 __device__ __forceinline__ uint4 tile_words(const SpTables& T, uint32_t q, uint32_t t) {
   uint4 w = __ldg(T.base + q);
-  for (uint32_t m = t, j = 0; m; m >>= 1, ++j)
-    if (m & 1u) w = xor4(w, __ldg(T.hi + (size_t)j * T.n_sub + q));
+  const uint4* h = T.hi + q;
+  // four set bits at a time, their loads in flight together
+  for (uint32_t m = t; m;) {
+    uint4 v[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      v[i] = make_uint4(0u, 0u, 0u, 0u);
+      if (m) v[i] = __ldg(h + (size_t)(__ffs(m) - 1) * T.n_sub);
+      m &= m - 1u;
+    }
+    w = xor4(w, xor4(xor4(v[0], v[1]), xor4(v[2], v[3])));
+  }
   return w;
 }
 
@@ -817,10 +827,9 @@ __global__ void __launch_bounds__(kSpThreads, 1) k_apply_h_sparse(const SparseAr
       }
     }
     __syncthreads();
-    if (a.partials && threadIdx.x < 2) {
-      double sum = 0.0;
-      for (int q = 0; q < NT / 32; ++q) sum += s_red[threadIdx.x][q];
-      a.partials[2u * t + threadIdx.x] = sum;
+    if (a.partials && warp < 2) {
+      const double sum = warp_sum(s_red[warp][lane]);
+      if (lane == 0) a.partials[2u * t + warp] = sum;
     }
     // then the whole tile out (zeros included) and the accumulator cleared
     for (uint32_t o = threadIdx.x; o < n_oct; o += NT) {

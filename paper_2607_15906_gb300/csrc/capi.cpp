@@ -81,7 +81,6 @@ int32_t* selected_ptr(Problem& p);
 int32_t* err_ptr(Problem& p);
 int dev_setup(Problem& p, void* psi, const double* d_theta, int n_ops, cudaStream_t st);
 int dev_taylor_chain(Problem& p, const int32_t* d_ops, int n_ops, void* psi, bool tracked, cudaStream_t st);
-int dev_apply_h(Problem& p, const void* psi, void* hpsi, bool energy, cudaStream_t st);
 int dev_norm(Problem& p, const void* psi, cudaStream_t st);
 int dev_pool_grads(Problem& p, const void* psi, const void* hpsi, double* d_grads, bool mask_current,
                    bool norm_current, cudaStream_t st);
@@ -535,7 +534,7 @@ int gocp_energy_grad(const gocp_problem* h, const int32_t* ops, const double* th
   } else {
     if ((rc = dev_setup(p, psi, d_theta, n_ops, st))) return rc;
     if ((rc = dev_taylor_chain(p, d_ops, n_ops, psi, true, st))) return rc;
-    if ((rc = dev_apply_h(p, psi, lam, true, st))) return rc;
+    if ((rc = dev_apply_h(p, psi, lam, true, st, true))) return rc;
     if (n_ops > 0 && (rc = dev_adjoint(p, d_ops, n_ops, psi, lam, d_dE, st))) return rc;
   }
   if (mem == GOCP_MEM_DEVICE) {
@@ -571,8 +570,8 @@ int gocp_adapt_step(const gocp_problem* h, const int32_t* ops, const double* the
   } else {
     if ((rc = dev_setup(p, psi, d_theta, n_ops, st))) return rc;
     if ((rc = dev_taylor_chain(p, d_ops, n_ops, psi, true, st))) return rc;
-    if ((rc = dev_apply_h(p, psi, hpsi, true, st))) return rc;
-    // the chain's octet mask, and <psi|psi> from the energy epilogue just run
+    if ((rc = dev_apply_h(p, psi, hpsi, true, st, true))) return rc;
+    // the chain's octet mask, and the amplitude list and <psi|psi> of the H psi just run
     if ((rc = dev_pool_grads(p, psi, hpsi, d_grads, true, true, st))) return rc;
   }
   int32_t* d_sel = mem == GOCP_MEM_DEVICE ? selected : selected_ptr(p);

@@ -656,10 +656,14 @@ int live_octets(const uint32_t* mask, int n, const LiveOctets& lv, cudaStream_t 
 // t.n_pieces must be > 0.  States whose nonzero amplitudes are at most the
 // fraction GOCP_SPARSE_FRAC (default 0.125, at most 0.25) of all take the
 // scatter kernel of apply_sparse.cu, the others the staged kernel; the
-// choice is made on the device from the count.  Defined in apply_tiled.cu.
+// choice is made on the device from the count.  mask_current: t.octmask already
+// marks every octet of psi that holds a nonzero amplitude.  Defined in
+// apply_tiled.cu.
 int tiled_apply_h(const DevTables& t, const LiveOctets& lv, int precision, int sm_count, const void* psi,
                   void* hpsi, double identity, double* partials, unsigned int* counter,
-                  unsigned int* tile_counter, double* scal, int32_t* err, cudaStream_t st);
+                  unsigned int* tile_counter, double* scal, int32_t* err, bool mask_current, cudaStream_t st);
+// Whether a tiled_apply_h call lists psi's nonzero amplitudes into lv.
+bool scatter_lists(const DevTables& t, const LiveOctets& lv);
 
 // Pieces the scatter kernel takes (four bytes of shared memory each); a
 // problem with more keeps every state on the staged kernel.

@@ -195,7 +195,9 @@ enum StageKind { STAGE_SETUP = 0, STAGE_FORWARD = 1, STAGE_ENERGY = 2, STAGE_BAC
 bool has_tiled_form(const Problem& p);
 // H psi (+ the energy into scalars_ptr(p): E, <psi|psi>, Re<psi|H'psi>) of a
 // full-layout problem on `st` (kernels.cu).
-int dev_apply_h(Problem& p, const void* psi, void* hpsi, bool energy, cudaStream_t st);
+// mask_current: the problem's octet mask already describes psi (a tracked chain of
+// a LUT pool just produced it), so psi is not read for it.
+int dev_apply_h(Problem& p, const void* psi, void* hpsi, bool energy, cudaStream_t st, bool mask_current = false);
 double* scalars_ptr(Problem& p);
 // Whether an item of this problem can take the on-chip stage `kind`
 // (STAGE_FORWARD_ALL: its state fits one block's shared memory;

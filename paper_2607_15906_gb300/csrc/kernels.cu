@@ -2030,7 +2030,7 @@ int build_scatter(int n, const std::vector<HLut<R>>& hl, const std::vector<uint3
       c.p.xhi = xhi;
       c.p.sub0 = s0;
       c.p.nsub = (uint16_t)std::min(max_sub, s1 - s0);
-      c.p.span = (uint16_t)(kind >= 2u ? 1u : std::max(1u, 4u / c.p.nsub));
+      c.p.span = (uint16_t)(kind >= 2u ? 1u : kind == 1u ? 2u : std::max(1u, 8u / c.p.nsub));
       c.p.kind = (uint16_t)kind;
       c.p.tab0 = (uint16_t)tab0;
       c.cost = each * c.p.nsub * c.p.span;
@@ -2110,7 +2110,13 @@ int build_scatter(int n, const std::vector<HLut<R>>& hl, const std::vector<uint3
           const double av = std::fabs((double)L.lut16[o]);
           if constexpr (sizeof(R) == 4) c.it.w = (float)av;
           else c.it.w = std::llround(std::ldexp(av, fd));
-          if (c.it.w != 0 && c.reduce()) cs.push_back(c);
+          // A weight whose every product rounds to zero is left out (the sums
+          // of a two-electron group's strings leave residues of 1e-17 where
+          // the exact coupling is zero): |w v| 2^F < 1/4 for complex64, where
+          // 2^F <= 2^30 / (2 dmax m) (see the kernel), and for complex128,
+          // where 2^F <= 2^62 / (2 hbound m), m the largest component.
+          const bool seen = sizeof(R) == 4 ? av > d.t.dmax * 0x1p-31 : av > d.t.hbound * 0x1p-63;
+          if (seen && c.reduce()) cs.push_back(c);
           left &= ~codes;
           found = true;
         }
@@ -3961,12 +3967,13 @@ int dev_taylor_chain(Problem& p, const int32_t* d_ops, int n_ops, void* psi, boo
 }
 
 template <typename R>
-static int launch_apply(Problem& p, const void* psi, void* hpsi, bool energy, cudaStream_t st) {
+static int launch_apply(Problem& p, const void* psi, void* hpsi, bool energy, bool mask_current, cudaStream_t st) {
   DeviceTables& d = *p.dev;
   if (d.t.n_pieces > 0) {
     ProfScope ps(GOCP_KERNEL_APPLY_H, st);
     return tiled_apply_h(d.t, d.live, p.precision, d.sm_count, psi, hpsi, p.identity, energy ? d.scratch : nullptr,
-                         d.counters + kMaxChunks, d.counters + kMaxChunks + 3, d.scalars, d.err, st);
+                         d.counters + kMaxChunks, d.counters + kMaxChunks + 3, d.scalars, d.err,
+                         mask_current && d.t.pool_lut, st);
   }
   const int grid = apply_grid(p.n_qubits);
   {
@@ -3979,9 +3986,9 @@ static int launch_apply(Problem& p, const void* psi, void* hpsi, bool energy, cu
   return cuda_status(cudaGetLastError(), "k_apply_h");
 }
 
-int dev_apply_h(Problem& p, const void* psi, void* hpsi, bool energy, cudaStream_t st) {
-  return p.precision == GOCP_C64 ? launch_apply<float>(p, psi, hpsi, energy, st)
-                                 : launch_apply<double>(p, psi, hpsi, energy, st);
+int dev_apply_h(Problem& p, const void* psi, void* hpsi, bool energy, cudaStream_t st, bool mask_current) {
+  return p.precision == GOCP_C64 ? launch_apply<float>(p, psi, hpsi, energy, mask_current, st)
+                                 : launch_apply<double>(p, psi, hpsi, energy, mask_current, st);
 }
 
 template <typename R>
@@ -4001,7 +4008,7 @@ int dev_norm(Problem& p, const void* psi, cudaStream_t st) {
 
 template <typename R>
 static int launch_pool_grads(Problem& p, const void* psi, const void* hpsi, double* d_grads, bool mask_current,
-                             cudaStream_t st) {
+                             bool list_current, cudaStream_t st) {
   DeviceTables& d = *p.dev;
   const int M = d.t.M;
   if (M == 0) return GOCP_OK;
@@ -4023,7 +4030,7 @@ static int launch_pool_grads(Problem& p, const void* psi, const void* hpsi, doub
       const uint64_t octets = 1ull << (p.n_qubits - 3);
       int lnbx = (int)std::max<uint64_t>(1, std::min<uint64_t>(64, (octets + kThreads * 64 - 1) / (kThreads * 64)));
       lnbx = std::max(1, std::min<int>(lnbx, (int)(d.scratch_doubles / ((size_t)nchunks * kOpsPerBlock))));
-      if (amps && (rc = amp_list(p.precision, psi, mask, p.n_qubits, d.live, st))) return rc;
+      if (amps && !(list_current && scatter_lists(d.t, d.live)) && (rc = amp_list(p.precision, psi, mask, p.n_qubits, d.live, st))) return rc;
       if ((rc = live_octets(mask, p.n_qubits, d.live, st))) return rc;
       {
         ProfScope ps(GOCP_KERNEL_POOL_GRAD, st, amps ? 2 : 1);
@@ -4068,8 +4075,9 @@ int dev_pool_grads(Problem& p, const void* psi, const void* hpsi, double* d_grad
     int rc = dev_norm(p, psi, st);   // <psi|psi> -> scalars[1]
     if (rc) return rc;
   }
-  return p.precision == GOCP_C64 ? launch_pool_grads<float>(p, psi, hpsi, d_grads, mask_current, st)
-                                 : launch_pool_grads<double>(p, psi, hpsi, d_grads, mask_current, st);
+  // with the norm from that call, its amplitude list is psi's too
+  return p.precision == GOCP_C64 ? launch_pool_grads<float>(p, psi, hpsi, d_grads, mask_current, norm_current, st)
+                                 : launch_pool_grads<double>(p, psi, hpsi, d_grads, mask_current, norm_current, st);
 }
 
 template <typename R>
