@@ -628,6 +628,23 @@ __global__ void __launch_bounds__(kSpThreads, 1) k_apply_h_sparse(const SparseAr
     // the claim is part `part` of output tile t: the part takes the tile's
     // unit batches part, part + K, part + 2K, ...
     const uint32_t t = claim / K, part = claim - t * K;
+    // A tile none of whose source tiles holds an amplitude (its own among them,
+    // for the diagonal) is all zero: no tables, no accumulator.  Few amplitudes
+    // in a large state leave most tiles so.
+    if (K == 1u) {
+      bool any = false;
+      for (uint32_t p = threadIdx.x; p < P && !any; p += NT) {
+        const uint32_t u = t ^ a.sp.piece[p].xhi;
+        any = a.toff[u + 1] != a.toff[u];
+      }
+      if (!__syncthreads_or(any || a.toff[t + 1] != a.toff[t])) {
+        float4* d4 = reinterpret_cast<float4*>(a.out + (size_t)t * kSpTile);
+        for (uint32_t q = threadIdx.x; q < n_oct * (8u * (uint32_t)sizeof(C_t<R>) / 16u); q += NT)
+          __stcs(d4 + q, make_float4(0.f, 0.f, 0.f, 0.f));
+        if (a.partials && threadIdx.x < 2) a.partials[2u * t + threadIdx.x] = 0.0;
+        continue;
+      }
+    }
     // Work units are (piece p, span of chunks): 32 span consecutive nonzero
     // amplitudes of p's source tile u = t ^ (x >> LB) against p's groups,
     // numbered piece by piece (s_pre: a block scan of the unit counts).
