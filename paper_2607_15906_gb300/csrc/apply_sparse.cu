@@ -39,11 +39,11 @@
 // from them are reproducible bit for bit from run to run.
 //
 // What bounds it (24 qubits, 233,867 nonzero amplitudes, 2.3e8 nonzero
-// products): instruction issue and the latency of the table reads, 54 % of the
-// issue slots busy with 7.2e8 warp instructions; the shared-memory atomics'
-// wavefronts take 0.37 ms.  2.29 -> 1.21 ms (complex64), 6.24 -> 2.0 ms
-// (complex128), 18.0 -> 10.4 ms at 28 qubits, against the kernel that tested
-// every pair.
+// products): the latency of the table reads and of a unit's start, with 54 % of
+// the issue slots busy (7e8 warp instructions); the shared-memory atomics'
+// wavefronts take 0.37 ms.  2.29 -> 1.1 ms (complex64), 6.2 -> 1.9 ms
+// (complex128), 18 -> 9 ms at 28 qubits (where the tables of 32,768 tiles are a
+// fifth), against the kernel that tested every pair.
 //
 // The kernel is launched with the staged one; each returns at once unless
 // the count of nonzero amplitudes selects it, so the choice needs no host
