@@ -342,8 +342,8 @@ __host__ __device__ constexpr int kRingAdd(int i) { return 24 + 8 * i; }
 constexpr int kRingWords = 48;
 
 // Words of a list chain's synchronisation (ChainList::sync), each in its own
-// 32-byte sector: arrivals at the grid barrier, a flag, one inbox length per
-// block.
+// 32-byte sector: arrivals at the grid barrier, a flag, one inbox record per
+// block (inbox.h).
 constexpr int kSyncBar = 0, kSyncFull = 8, kSyncInbox = 16, kSyncWords = 16 + 8 * 256;
 
 struct ChainList {

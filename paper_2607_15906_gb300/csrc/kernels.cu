@@ -25,6 +25,7 @@
 #include <cooperative_groups.h>
 
 #include "device.cuh"
+#include "inbox.h"
 #include "internal.h"
 
 namespace gocp {
@@ -3221,7 +3222,7 @@ __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.w
 // entries of a share in shared memory (at most kListSmem).  A list
 // that is incomplete, or an inbox that overflows, is given up for the
 // operator's enumerated pairs (full).  tb.cl.sync: the barrier's count, the
-// full flag and the inbox lengths, zero at the start.  CLUSTER: the blocks are
+// full flag and the inbox records (inbox.h), zero at the start.  CLUSTER: the blocks are
 // one thread-block cluster and take its hardware barrier; else the barrier is
 // a count in global memory whose wait gives up after wait_ns (recorded in err,
 // the results are then undefined).
@@ -3236,6 +3237,7 @@ k_chain_list(DevTables tb, const int32_t* ops, const double* coefs, int n_ops, C
   uint32_t* queue = list + kListSmem;
   ListStep<R>* sd = reinterpret_cast<ListStep<R>*>(queue + kListQueue * (kSmemThreads / 32));
   __shared__ uint32_t s_in, s_full, s_n;   // inbox length; see full; entries of the share in list
+  __shared__ uint32_t s_sent[2];           // entries sent here in even and in odd steps, as last read
   __shared__ int s_abort;
   __shared__ Sum s_sum[kSmemThreads / 32];
   const uint32_t G = gridDim.x, rank = blockIdx.x;
@@ -3271,7 +3273,7 @@ k_chain_list(DevTables tb, const int32_t* ops, const double* coefs, int n_ops, C
   const uint32_t n_far = n_first - n_list;
   if (threadIdx.x == 0) {
     s_n = n_list;
-    s_in = 0u;
+    s_in = s_sent[0] = s_sent[1] = 0u;
     s_full = full;
     s_abort = 0;
   }
@@ -3336,12 +3338,14 @@ k_chain_list(DevTables tb, const int32_t* ops, const double* coefs, int n_ops, C
       if (warp == 0) {
         if (!CLUSTER && lane == 0 && !grid_wait(bar, (uint32_t)i * G, wait_ns, err)) s_abort = 1;
         __syncwarp();
-        const uint32_t got = min(__ldcg(in_lens + 8u * rank), seg), over = __ldcg(full_flag);
+        const uint32_t sent = __ldcg(in_lens + 8u * rank + inbox_read_word(i)), over = __ldcg(full_flag);
         const uint32_t q = in_len + lane, early = q < seg ? __ldcg(mine_in + q) : 0u;
+        const uint32_t got = inbox_length(sent, s_sent[i & 1], seg);
         if (n_far == 0u && in_base == in_len && q < got && n_list + lane < cap) list[n_list + lane] = early;
         if (lane == 0) {
           s_in = got;
-          if (over) s_full = 1u;
+          s_sent[(i + 1) & 1] = sent;
+          if (full_heeded(over, i)) s_full = 1u;
         }
       }
       __syncthreads();
@@ -3421,9 +3425,10 @@ k_chain_list(DevTables tb, const int32_t* ops, const double* coefs, int n_ops, C
           }
         }
         const uint32_t to = ((other * 0x9E3779B1u) >> 12) % G;
-        const uint32_t pos = atomicAdd(in_lens + 8u * to, 1u);
+        const uint32_t pos = atomicAdd(in_lens + 8u * to + kInboxNext, 1u);
+        atomicAdd(in_lens + 8u * to + inbox_send_word(i), 1u);
         if (pos < seg) __stcg(inbox + (size_t)to * seg + pos, other);
-        else atomicOr(full_flag, 1u);   // no room: pairs are enumerated from the next step on
+        else atomicCAS(full_flag, 0u, full_mark(i));   // no room: pairs are enumerated from the next step on
       };
       if (!full) {
         for (;;) {
@@ -3682,6 +3687,7 @@ int launch_list_chain(Problem& p, int blocks, bool back, const int32_t* d_ops, i
   uint64_t wait = chain_wait_ns();
   uint32_t cap = kListSmem;
   if (const char* v = std::getenv("GOCP_LIST_SHARE")) cap = (uint32_t)std::min(std::max(std::atoi(v), 64), (int)kListSmem);
+  if (const char* v = std::getenv("GOCP_LIST_INBOX")) seg = std::min(seg, (uint32_t)std::max(std::atoi(v), 1));
   void* args[] = {&tb, &d_ops, &coefs, &n, &ps, &ls, &mk, &ref, &slot, &inbox, &seg, &dpart, &err, &cap, &wait};
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)blocks, 1, 1);
