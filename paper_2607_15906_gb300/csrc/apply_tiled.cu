@@ -36,6 +36,7 @@
 
 #include "device.cuh"
 #include "internal.h"
+#include "parts.h"
 
 namespace gocp {
 
@@ -347,7 +348,7 @@ struct TiledArgs {
   // adds them up (K > 1)
   int K;
   C_t<R>* extra;
-  uint16_t pbeg[kTiledParts + 1];
+  uint32_t pbeg[kTiledParts + 1];
 };
 
 template <typename R>
@@ -734,18 +735,6 @@ double sparse_frac() {
   return f < 0.0 ? 0.0 : (f > 0.25 ? 0.25 : f);
 }
 
-// First piece of part q of K: the pieces cut at equal shares of their bytes,
-// at least one piece to a part (K <= n_pieces).
-uint16_t tiled_cut(const DevTables& t, int q, int K) {
-  const std::vector<uint32_t>& off = *t.piece_off;
-  const int P = t.n_pieces;
-  if (q >= K) return (uint16_t)P;
-  const uint64_t want = (uint64_t)off[P] * (uint64_t)q / (uint64_t)K;
-  int p = (int)(std::lower_bound(off.begin(), off.end(), (uint32_t)want) - off.begin());
-  p = std::max(p, q);
-  return (uint16_t)std::min(p, P - (K - q));
-}
-
 template <typename R>
 int launch_tiled(const DevTables& t, const LiveOctets& lv, int sm_count, const void* psi, void* hpsi,
                  double identity, double* partials, unsigned int* counter, unsigned int* tile_counter, double* scal,
@@ -851,7 +840,7 @@ int launch_tiled(const DevTables& t, const LiveOctets& lv, int sm_count, const v
   }
   a.K = K;
   a.extra = reinterpret_cast<C_t<R>*>(lv.gacc);
-  for (int q = 0; q <= K; ++q) a.pbeg[q] = tiled_cut(t, q, K);
+  tiled_cuts(t.piece_off->data(), t.n_pieces, K, a.pbeg);
   const int per_sm = sizeof(R) == 4 ? GOCP_TILED_MINB_C64 : 1;
   const int grid = (int)std::min<uint64_t>(ntiles * K, sms * per_sm);
   auto kern = K > 1 ? k_apply_h_tiled<R, true> : k_apply_h_tiled<R, false>;
