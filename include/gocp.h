@@ -210,8 +210,10 @@ int gocp_reference_state(const gocp_problem* p, void* psi, void* stream);
  * per step, "block" the one-block form where it fits, else that, "all" also a
  * cluster's shared memory for states up to 2 MiB, "list" the list form
  * for every problem (GOCP_LIST_SHARE caps the entries a block of it keeps in
- * shared memory, GOCP_LIST_INBOX those that others may send it).  Every form
- * gives the same state bit for bit. */
+ * shared memory, GOCP_LIST_INBOX those that others may send it).  Where the
+ * driver refuses a launch whose blocks wait for one another (GOCP_CHAIN_REFUSE=1:
+ * as if it did), the chain takes a launch per step.  Every form gives the same
+ * state bit for bit. */
 int gocp_prepare_state(const gocp_problem* p, const int32_t* ops, const double* theta, int n_ops,
                        int mem, void* psi, void* stream);
 

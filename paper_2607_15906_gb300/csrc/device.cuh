@@ -732,6 +732,8 @@ int ensure_stage(Problem& p, int n_ops);
 double* dpart_ptr(Problem& p);          // stage capacity x at least the SM count
 bool chain_forms_default();             // GOCP_ONCHIP_CHAINS is unset
 uint64_t chain_wait_ns();               // limit of a wait between the blocks of a chain
+constexpr int kChainRefused = 1;        // beside the GOCP_ codes: the chain's one launch was refused, nothing ran
+int launch_together(const cudaLaunchConfig_t& cfg, const void* kernel, void** args, bool* refused);
 int dtheta_reduce(Problem& p, int blocks, int n_ops, double* d_dE, cudaStream_t st);
 double* scalars_ptr(Problem& p);
 int32_t* err_ptr(Problem& p);

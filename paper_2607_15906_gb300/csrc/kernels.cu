@@ -3667,6 +3667,23 @@ int dtheta_reduce(Problem& p, int blocks, int n_ops, double* d_dE, cudaStream_t 
   return cuda_status(cudaGetLastError(), "k_dtheta_reduce");
 }
 
+// Launches blocks that wait for one another.  *refused: they cannot all be
+// resident here (a context with fewer SMs than the device names, or a driver
+// without such launches), nothing ran, and the caller takes a launch per step;
+// GOCP_CHAIN_REFUSE=1 answers so without asking.
+int launch_together(const cudaLaunchConfig_t& cfg, const void* kernel, void** args, bool* refused) {
+  const char* ev = std::getenv("GOCP_CHAIN_REFUSE");
+  const cudaError_t e =
+      ev && ev[0] == '1' ? cudaErrorCooperativeLaunchTooLarge : cudaLaunchKernelExC(&cfg, kernel, args);
+  *refused = e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorLaunchOutOfResources ||
+             e == cudaErrorInvalidConfiguration || e == cudaErrorNotSupported;
+  if (*refused) {
+    cudaGetLastError();
+    return GOCP_OK;
+  }
+  return cuda_status(e, "chain launch");
+}
+
 template <typename R>
 int launch_list_chain(Problem& p, int blocks, bool back, const int32_t* d_ops, int n_ops, void* psi, void* lam,
                       double* d_dE, cudaStream_t st) {
@@ -3710,8 +3727,10 @@ int launch_list_chain(Problem& p, int blocks, bool back, const int32_t* d_ops, i
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   ProfScope prof(back ? GOCP_KERNEL_ADJOINT : GOCP_KERNEL_TAYLOR, st, 1);
-  int rc = cuda_status(cudaLaunchKernelExC(&cfg, k, args), "list chain launch");
+  bool refused = false;
+  int rc = launch_together(cfg, k, args, &refused);
   if (rc) return rc;
+  if (refused) return kChainRefused;
   count_launches(1);
   return back ? dtheta_reduce(p, blocks, n_ops, d_dE, st) : GOCP_OK;
 }
@@ -3943,8 +3962,10 @@ static int launch_taylor_chain(Problem& p, const int32_t* d_ops, int n_ops, void
     }
   }
   if (tracked && n_ops > 1)
-    if (const int lb = list_chain_blocks<R>(p, n_ops, false))   // over the nonzero amplitudes, in one launch
-      return launch_list_chain<R>(p, lb, false, d_ops, n_ops, psi, nullptr, nullptr, st);
+    if (const int lb = list_chain_blocks<R>(p, n_ops, false)) {   // over the nonzero amplitudes, in one launch
+      const int rc = launch_list_chain<R>(p, lb, false, d_ops, n_ops, psi, nullptr, nullptr, st);
+      if (rc != kChainRefused) return rc;
+    }
   const int grid = d.t.pool_lut ? grid_for((uint64_t)d.t.penum_max, d.sm_count, kChainBlocksPerSm)
                                 : grid_for(1ull << (p.n_qubits - 1), d.sm_count, 8);
   uint32_t* mask = tracked && d.t.pool_lut ? d.t.octmask : nullptr;
@@ -4137,8 +4158,10 @@ static int launch_adjoint(Problem& p, const int32_t* d_ops, int n_ops, void* psi
                        (n_ops - 1) % 3, st)))
     return rc;
   count_launches(1);   // k_residual (and k_octet_mask counts itself)
-  if (const int lb = mask && d.t.cl.list ? list_chain_blocks<R>(p, n_ops, true) : 0)
-    return launch_list_chain<R>(p, lb, true, d_ops, n_ops, psi, lam, d_dE, st);
+  if (const int lb = mask && d.t.cl.list ? list_chain_blocks<R>(p, n_ops, true) : 0) {
+    rc = launch_list_chain<R>(p, lb, true, d_ops, n_ops, psi, lam, d_dE, st);
+    if (rc != kChainRefused) return rc;
+  }
   double* dpart = d.t.pool_lut ? d.dpart : nullptr;
   DevTables tb = d.t;
   const double* coefs = d.coefs;

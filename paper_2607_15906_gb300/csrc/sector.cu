@@ -717,16 +717,20 @@ int launch_sec_chain(Problem& p, int blocks, bool back, const int32_t* d_ops, in
   cfg.numAttrs = 1;
   ProfScope prof(back ? GOCP_KERNEL_ADJOINT : GOCP_KERNEL_TAYLOR, st, 1);
   const void* k = back ? (const void*)k_sec_chain<R, true> : (const void*)k_sec_chain<R, false>;
-  const int rc = cuda_status(cudaLaunchKernelExC(&cfg, k, args), "sector chain launch");
+  bool refused = false;
+  const int rc = launch_together(cfg, k, args, &refused);
   if (rc) return rc;
+  if (refused) return kChainRefused;
   count_launches(1);
   return back ? dtheta_reduce(p, blocks, n_ops, d_dE, st) : GOCP_OK;
 }
 
 template <typename R>
 int sec_taylor_t(Problem& p, const int32_t* d_ops, int n_ops, void* psi, cudaStream_t st) {
-  if (const int b = sec_chain_blocks(p, n_ops))
-    return launch_sec_chain<R>(p, b, false, d_ops, n_ops, psi, nullptr, nullptr, st);
+  if (const int b = sec_chain_blocks(p, n_ops)) {
+    const int rc = launch_sec_chain<R>(p, b, false, d_ops, n_ops, psi, nullptr, nullptr, st);
+    if (rc != kChainRefused) return rc;
+  }
   const int grid = pair_grid(p, 8);
   SecDev sd = p.sec->s;
   DevTables tb = dev_tables(p);
@@ -778,8 +782,10 @@ int sec_adjoint_t(Problem& p, const int32_t* d_ops, int n_ops, void* psi, void* 
   k_sec_residual<R><<<grid_rows(D, sm_of(p), 8), kSecThreads, 0, st>>>((const C_t<R>*)psi, (C_t<R>*)lam, D,
                                                                        scalars_ptr(p), dev_tables(p).cl.sync);
   count_launches(1);   // k_sec_residual
-  if (const int b = sec_chain_blocks(p, n_ops))
-    return launch_sec_chain<R>(p, b, true, d_ops, n_ops, psi, lam, d_dE, st);
+  if (const int b = sec_chain_blocks(p, n_ops)) {
+    const int rc = launch_sec_chain<R>(p, b, true, d_ops, n_ops, psi, lam, d_dE, st);
+    if (rc != kChainRefused) return rc;
+  }
   const int grid = std::min<int>(pair_grid(p, 2), (int)nd);
   SecDev sd = p.sec->s;
   DevTables tb = dev_tables(p);
