@@ -298,7 +298,8 @@ int gocp_energy_static(const gocp_problem* p, const void* psi, void* hpsi, doubl
  * once when it is 0; the H psi and energy of that call are then undefined,
  * later calls are not affected).  Bit 2: a wait between the blocks of a chain
  * gave up (see gocp_prepare_state; the state, or dE, of that call is then
- * undefined).  Synchronises `stream`. */
+ * undefined; gocp_energy_grad and gocp_adapt_step with host arrays also return
+ * GOCP_ETIMEDOUT).  Synchronises `stream`. */
 int gocp_device_errors(const gocp_problem* p, int* flags, void* stream);
 
 /* ---------------------------------------------------------------- serving */

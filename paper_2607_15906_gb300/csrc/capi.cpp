@@ -114,6 +114,14 @@ int check_mem(int mem) {
   return GOCP_OK;
 }
 
+// Status of a call's chains, from the scalars it read back.
+int chain_finished(const double* scal) {
+  uint64_t w;
+  std::memcpy(&w, scal + kScalGaveUp, sizeof(w));
+  if (!w) return GOCP_OK;
+  return fail(GOCP_ETIMEDOUT, "a wait between the blocks of a chain ran out; the results are undefined");
+}
+
 size_t state_dim(const Problem& p) { return p.sector ? (size_t)p.sector_dim : (size_t)1 << p.n_qubits; }
 
 size_t state_bytes(const Problem& p) { return state_dim(p) * (p.precision == GOCP_C64 ? 8u : 16u); }
@@ -540,11 +548,14 @@ int gocp_energy_grad(const gocp_problem* h, const int32_t* ops, const double* th
   if (mem == GOCP_MEM_DEVICE) {
     return cuda_status(cudaMemcpyAsync(E, scalars_ptr(p), sizeof(double), cudaMemcpyDeviceToDevice, st), "copy E");
   }
-  if ((rc = cuda_status(cudaMemcpyAsync(E, scalars_ptr(p), sizeof(double), cudaMemcpyDeviceToHost, st), "copy E")))
+  double scal[kScalCount];
+  if ((rc = cuda_status(cudaMemcpyAsync(scal, scalars_ptr(p), sizeof(scal), cudaMemcpyDeviceToHost, st), "copy E")))
     return rc;
   if (n_ops > 0 && (rc = cuda_status(cudaMemcpyAsync(dE, d_dE, n_ops * sizeof(double), cudaMemcpyDeviceToHost, st), "copy dE")))
     return rc;
-  return cuda_status(cudaStreamSynchronize(st), "synchronise");
+  if ((rc = cuda_status(cudaStreamSynchronize(st), "synchronise"))) return rc;
+  *E = scal[0];
+  return chain_finished(scal);
 }
 
 int gocp_adapt_step(const gocp_problem* h, const int32_t* ops, const double* theta, int n_ops,
@@ -579,11 +590,15 @@ int gocp_adapt_step(const gocp_problem* h, const int32_t* ops, const double* the
   if (mem == GOCP_MEM_DEVICE) {
     return cuda_status(cudaMemcpyAsync(out_e, scalars_ptr(p), 2 * sizeof(double), cudaMemcpyDeviceToDevice, st), "copy E");
   }
-  if ((rc = cuda_status(cudaMemcpyAsync(out_e, scalars_ptr(p), 2 * sizeof(double), cudaMemcpyDeviceToHost, st), "copy E")) ||
+  double scal[kScalCount];
+  if ((rc = cuda_status(cudaMemcpyAsync(scal, scalars_ptr(p), sizeof(scal), cudaMemcpyDeviceToHost, st), "copy E")) ||
       (rc = cuda_status(cudaMemcpyAsync(grads, d_grads, p.pool.size() * sizeof(double), cudaMemcpyDeviceToHost, st), "copy grads")) ||
       (rc = cuda_status(cudaMemcpyAsync(selected, d_sel, sizeof(int32_t), cudaMemcpyDeviceToHost, st), "copy selection")))
     return rc;
-  return cuda_status(cudaStreamSynchronize(st), "synchronise");
+  if ((rc = cuda_status(cudaStreamSynchronize(st), "synchronise"))) return rc;
+  out_e[0] = scal[0];
+  out_e[1] = scal[1];
+  return chain_finished(scal);
 }
 
 int gocp_device_errors(const gocp_problem* h, int* flags, void* stream) {

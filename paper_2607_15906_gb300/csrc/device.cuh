@@ -56,8 +56,8 @@ __device__ __forceinline__ void chain_step_begin() {
 // Barrier between the blocks of a cooperative launch: a count in global memory
 // (zero at the launch).  grid_arrive by one thread after a block barrier, so
 // that the block's writes come before it; grid_wait by one thread before one,
-// false (recorded in err) when the count has not reached `want` after wait_ns
-// (0: at once).
+// false (recorded in err, and in gave_up for the call that waits for its results)
+// when the count has not reached `want` after wait_ns (0: at once).
 constexpr int32_t kErrChainTimeout = 4;
 __device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
   uint32_t v;
@@ -67,7 +67,8 @@ __device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
 __device__ __forceinline__ void grid_arrive(uint32_t* bar) {
   asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
 }
-__device__ __forceinline__ bool grid_wait(const uint32_t* bar, uint32_t want, uint64_t wait_ns, int32_t* err) {
+__device__ __forceinline__ bool grid_wait(const uint32_t* bar, uint32_t want, uint64_t wait_ns, int32_t* err,
+                                          uint32_t* gave_up) {
   uint64_t t0, t1;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
   for (uint32_t spin = 1; wait_ns != 0; ++spin) {
@@ -77,6 +78,7 @@ __device__ __forceinline__ bool grid_wait(const uint32_t* bar, uint32_t want, ui
     if (t1 - t0 > wait_ns) break;
   }
   atomicOr(err, kErrChainTimeout);
+  *gave_up = 1u;
   return false;
 }
 
@@ -351,6 +353,7 @@ struct ChainList {
   uint32_t* amask = nullptr;
   uint32_t* cnt = nullptr;
   uint32_t* sync = nullptr;   // zeroed where a chain's initial list is written
+  uint32_t* gave_up = nullptr;   // a wait of this call's chains gave up; zeroed by the set-up
   uint32_t cap = 0;
 };
 

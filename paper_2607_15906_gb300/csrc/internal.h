@@ -198,7 +198,10 @@ bool has_tiled_form(const Problem& p);
 // mask_current: the problem's octet mask already describes psi (a tracked chain of
 // a LUT pool just produced it), so psi is not read for it.
 int dev_apply_h(Problem& p, const void* psi, void* hpsi, bool energy, cudaStream_t st, bool mask_current = false);
+// [0] E, [1] <psi|psi>, [2] Re<psi|H'psi>, [kScalGaveUp] not zero: a wait between
+// the blocks of the present call's chains gave up.
 double* scalars_ptr(Problem& p);
+constexpr int kScalGaveUp = 3, kScalCount = 4;
 // Whether an item of this problem can take the on-chip stage `kind`
 // (STAGE_FORWARD_ALL: its state fits one block's shared memory;
 // STAGE_BACKWARD_ALL: its two states do).

@@ -136,8 +136,10 @@ k_setup(C_t<R>* psi, int n, uint64_t index, const double* theta, int n_ops, doub
         cl.cnt[kRingAdd(2)] = 0u;
         cl.cnt[kRingAdd(0)] = 0u;
       }
-      if (blockIdx.x == 0)
+      if (blockIdx.x == 0) {
         for (int w = threadIdx.x; w < kSyncWords; w += kThreads) cl.sync[w] = 0u;
+        if (threadIdx.x == 0) *cl.gave_up = 0u;
+      }
     }
   }
 }
@@ -2921,6 +2923,7 @@ int upload_problem(Problem& p) {
   if ((rc = dalloc(*d, &d->scratch, need, bytes))) return rc;
   if ((rc = dalloc(*d, &d->counters, kMaxChunks + 8, bytes))) return rc;
   if ((rc = dalloc(*d, &d->scalars, 16, bytes))) return rc;
+  d->t.cl.gave_up = reinterpret_cast<uint32_t*>(d->scalars + kScalGaveUp);
   if ((rc = dalloc(*d, &d->err, 1, bytes))) return rc;
   if ((rc = dalloc(*d, &d->selected, 1, bytes))) return rc;
   if ((rc = dalloc(*d, &d->grads, std::max(M, 1), bytes))) return rc;
@@ -3336,7 +3339,7 @@ k_chain_list(DevTables tb, const int32_t* ops, const double* coefs, int n_ops, C
       // same round trip, the first 32 entries it may have gained
       if constexpr (CLUSTER) cluster_wait();
       if (warp == 0) {
-        if (!CLUSTER && lane == 0 && !grid_wait(bar, (uint32_t)i * G, wait_ns, err)) s_abort = 1;
+        if (!CLUSTER && lane == 0 && !grid_wait(bar, (uint32_t)i * G, wait_ns, err, tb.cl.gave_up)) s_abort = 1;
         __syncwarp();
         const uint32_t sent = __ldcg(in_lens + 8u * rank + inbox_read_word(i)), over = __ldcg(full_flag);
         const uint32_t q = in_len + lane, early = q < seg ? __ldcg(mine_in + q) : 0u;

@@ -71,8 +71,9 @@ __device__ __forceinline__ void kahan(R& s, R& c, R v) {
 // psi = row ref; block 0 also writes coefs[6j + m] = theta_j^m / m!.
 template <typename R>
 __global__ void __launch_bounds__(kSecThreads)
-k_sec_setup(C_t<R>* psi, int32_t D, int32_t ref, const double* theta, int n_ops, double* coefs, uint32_t* sync) {
-  if (sync && blockIdx.x == 0 && threadIdx.x == 0) sync[kSyncBar] = 0u;   // for the chain that follows
+k_sec_setup(C_t<R>* psi, int32_t D, int32_t ref, const double* theta, int n_ops, double* coefs, uint32_t* sync,
+            uint32_t* gave_up) {
+  if (sync && blockIdx.x == 0 && threadIdx.x == 0) sync[kSyncBar] = *gave_up = 0u;   // for the chain that follows
   if (psi)
     for (int32_t r = blockIdx.x * kSecThreads + threadIdx.x; r < D; r += gridDim.x * kSecThreads)
       psi[r] = cmake<R>(r == ref ? R(1) : R(0), R(0));
@@ -517,7 +518,7 @@ k_sec_chain(SecDev s, DevTables tb, const uint2* __restrict__ pairs, const int64
 #pragma unroll
     for (int m = 0; m < 6; ++m) c[m] = D.c[m];
     if (i > 0 && G > 1u) {
-      if (threadIdx.x == 0 && !grid_wait(bar, (uint32_t)i * G, wait_ns, err)) s_abort = 1;
+      if (threadIdx.x == 0 && !grid_wait(bar, (uint32_t)i * G, wait_ns, err, tb.cl.gave_up)) s_abort = 1;
       __syncthreads();
       if (s_abort) return;
     }
@@ -1013,10 +1014,10 @@ int sec_setup(Problem& p, void* psi, const double* d_theta, int n_ops, void* str
   const int grid = psi ? grid_rows(p.sector_dim, sm_of(p), 8) : 1;
   if (p.precision == GOCP_C64)
     k_sec_setup<float><<<grid, kSecThreads, 0, st>>>((float2*)psi, p.sec->s.D, p.sec->ref_row, d_theta, n_ops,
-                                                     coefs_ptr(p), dev_tables(p).cl.sync);
+                                                     coefs_ptr(p), dev_tables(p).cl.sync, dev_tables(p).cl.gave_up);
   else
     k_sec_setup<double><<<grid, kSecThreads, 0, st>>>((double2*)psi, p.sec->s.D, p.sec->ref_row, d_theta, n_ops,
-                                                      coefs_ptr(p), dev_tables(p).cl.sync);
+                                                      coefs_ptr(p), dev_tables(p).cl.sync, dev_tables(p).cl.gave_up);
   count_launches(1);
   return cuda_status(cudaGetLastError(), "k_sec_setup");
 }
