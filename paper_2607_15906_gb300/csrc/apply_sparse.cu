@@ -425,10 +425,10 @@ __device__ __forceinline__ void sp_tab_items(const SpTab<R>* __restrict__ tab, c
       q += (__popc((kk ^ h.y) & __ldg(T.ry + r)) & 1) ? -v : v;
     }
     typename SpVal<R>::T d;
-    if constexpr (sizeof(R) == 4) d = (float)q * T.tscale;
+    if constexpr (sizeof(R) == 4) d = (float)q * __uint_as_float(h.x & 0xFFFF0000u);
     else d = q;
     d = sp_signed(d, sg << g);
-    const uint32_t at = acc_s + ((4u * klow) ^ h.x);
+    const uint32_t at = acc_s + ((4u * klow) ^ (h.x & 0xFFFFu));
     fx_put<SPLIT, kRe>(at, sp_product(d, vx));
     if (cplx) fx_put<SPLIT, kIm>(at, sp_product(d, vy));
   }

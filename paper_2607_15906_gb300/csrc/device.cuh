@@ -252,7 +252,7 @@ constexpr int kSpLB = 13;
 constexpr uint32_t kSpTile = 1u << kSpLB;
 constexpr int kSpCases = 32;
 template <typename R> struct SpWeight;
-template <> struct SpWeight<float> { using T = int32_t; };      // round(w 2^Ft)
+template <> struct SpWeight<float> { using T = int32_t; };      // round(w 2^Ft), Ft the group's
 template <> struct SpWeight<double> { using T = long long; };   // round(w 2^Fd)
 struct __align__(16) SpHead {
   uint4 ta[32], tb[16], tc[16];   // x, y, z: the parities p0, p1, p2; w: the sign
@@ -270,13 +270,17 @@ template <> struct __align__(16) SpItem<double> { long long w; uint32_t xo, pad;
 // index, x folded in), in fixed point: fa, fb, fc; those with y among the
 // tile's bits are summed once per tile (hy, hw; the constant f0 with them);
 // the others stay a list (ry over all bits, rw).  Integer sums, so their
-// order does not matter.
+// order does not matter.  complex64: Ft = 30 - e with the group's sum of
+// magnitudes < 2^e, so that a weight keeps the bits it has in FP32 down to 2^-6
+// of that sum, whatever the other groups' size.  xo: the offset 4 (x mod
+// 2^kSpLB), and for complex64 the upper half of the float 2^-Ft above it.
 template <typename R>
 struct __align__(16) SpTab {
   using W = typename SpWeight<R>::T;
   W fa[32], fb[16], fc[16];
   uint32_t xo, x, rb, re;
 };
+static_assert(4u * (kSpTile - 1u) <= 0xFFFFu, "an offset leaves the upper half of the word free");
 // The per-tile part of a term group: f0 and the terms [hb, he) of hy, hw.
 template <typename R>
 struct __align__(8) SpTabTile {
@@ -317,7 +321,6 @@ struct SpTables {
   const SpListGroup* list = nullptr;
   const uint32_t* lz = nullptr;     // their terms: masks, weights (complex64: float, complex128: round(w 2^Fd))
   const void* lw = nullptr;
-  float tscale = 1.f;               // 2^-Ft
   double wscale = 1.0;              // 2^(63 - Fd): takes an amplitude scaled by 2^F to the integer whose product
                                     // with a weight, shifted right by 63, is the product at 2^F
   // the diagonal group and the identity (mask 0), weights as round(w 2^Fg),

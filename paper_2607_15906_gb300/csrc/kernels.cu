@@ -2151,13 +2151,13 @@ int build_scatter(int n, const std::vector<HLut<R>>& hl, const std::vector<uint3
     uint32_t x, zc, delta, neg;
     std::vector<uint32_t> y;
     std::vector<double> w;
+    int ft;   // the scale of its weights, 2^ft
   };
   std::vector<TabGroup> tabs;
   std::vector<SpListGroup> list;
   std::vector<uint32_t> lz;
   std::vector<double> lw;
   std::vector<uint32_t> list_hi;
-  double tmax = 0.0;   // the largest sum of |w| of a table group
   for (size_t g = 0; g < gx.size(); ++g) {
     const auto pr = paired_terms<R>(tz, tw, goff[g], gmid[g], goff[g + 1]);
     std::vector<uint32_t> z;
@@ -2181,14 +2181,15 @@ int build_scatter(int n, const std::vector<HLut<R>>& hl, const std::vector<uint3
         }
       }
     if (real && 2 * best >= z.size() && !z.empty() && tabs.size() < kSpMaxTab) {
-      TabGroup t{gx[g], z[at], pr.delta, pr.neg, {}, {}};
+      TabGroup t{gx[g], z[at], pr.delta, pr.neg, {}, {}, fd};
       double sum = 0.0;
       for (size_t q = 0; q < z.size(); ++q) {
         t.y.push_back(z[q] ^ z[at]);
         t.w.push_back(pr.delta ? 2.0 * w[q] : w[q]);
         sum += std::fabs(t.w.back());
       }
-      tmax = std::max(tmax, sum);
+      // (2^-ft is a normal float)
+      if (sizeof(R) == 4) t.ft = std::max(-126, std::min(126, 30 - log2_above(sum)));
       tabs.push_back(std::move(t));
     } else {
       SpListGroup L;
@@ -2203,8 +2204,6 @@ int build_scatter(int n, const std::vector<HLut<R>>& hl, const std::vector<uint3
       list.push_back(L);
     }
   }
-  const int ft = sizeof(R) == 4 ? 30 - log2_above(tmax) : fd;
-  auto fix = [&](double w) { return (W)std::llround(std::ldexp(w, ft)); };
   std::stable_sort(tabs.begin(), tabs.end(),
                    [](const TabGroup& a, const TabGroup& b) { return (a.x >> kSpLB) < (b.x >> kSpLB); });
   std::vector<SpTab<R>> tab;
@@ -2230,11 +2229,17 @@ int build_scatter(int n, const std::vector<HLut<R>>& hl, const std::vector<uint3
       std::memset(&tt, 0, sizeof(tt));
       tt.hb = (uint32_t)hy.size();
       S.xo = 4u * (t.x & kLow);
+      if (sizeof(R) == 4) {
+        const float scale = (float)std::ldexp(1.0, -t.ft);
+        uint32_t up;
+        std::memcpy(&up, &scale, sizeof(up));   // a power of two: the lower half is zero
+        S.xo |= up;
+      }
       S.x = t.x;
       S.rb = (uint32_t)ry.size();
       for (size_t q = 0; q < t.y.size(); ++q) {
         const uint32_t y = t.y[q];
-        const W wq = fix(t.w[q]);
+        const W wq = (W)std::llround(std::ldexp(t.w[q], t.ft));
         const int rg = range_of(y);
         auto spread = [&](W* f, int size, int from) {   // over the source bits
           for (int v = 0; v < size; ++v) {
@@ -2319,7 +2324,6 @@ int build_scatter(int n, const std::vector<HLut<R>>& hl, const std::vector<uint3
   T.n_pieces = (int)sp.size();
   T.n_sub = (uint32_t)head.size();
   T.n_tab = (uint32_t)tile.size();
-  T.tscale = (float)std::ldexp(1.0, -ft);
   T.wscale = std::ldexp(1.0, 63 - fd);
   T.dscale = std::ldexp(1.0, 63 - fg);
   // one device buffer for all of it: an allocation and a copy each would cost
