@@ -231,8 +231,9 @@ int gocp_taylor_step(const gocp_problem* p, int op, double theta, void* psi, voi
  * lets up to 64 blocks share a tile (GOCP_SCATTER_PARTS, environment, caps
  * that number; 1 = one block per tile); the result does not depend on it.
  * complex64 adds each fixed-point product as two independent 32-bit
- * counts when H has fewer than 57344 off-diagonal x-groups
- * (GOCP_SCATTER_SPLIT=0: as one 64-bit add with a carry); same result. */
+ * counts when H has fewer than 57344 off-diagonal x-groups and no constant or
+ * diagonal beyond 2^15 times its couplings (GOCP_SCATTER_SPLIT=0: as one 64-bit
+ * add with a carry); same result. */
 int gocp_apply_h(const gocp_problem* p, const void* psi, void* hpsi, void* stream);
 
 /* hpsi <- H psi, and out[0] = E = Re<psi|H psi>/<psi|psi> (Eq. 1),

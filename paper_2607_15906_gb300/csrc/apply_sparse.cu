@@ -249,9 +249,9 @@ k_tile_offsets(const uint32_t* __restrict__ idx, const uint32_t* __restrict__ le
 // sum is exact integer arithmetic: the same in any order of the atomics,
 // and the result is bit-for-bit reproducible.  F is chosen per call so that
 // the sum of the magnitudes of all contributions to one output component --
-// at most hbound x 2 max(|Re psi|, |Im psi|) -- stays below 2^62 (complex64:
-// 2^46): no partial sum can overflow.  For complex64, F also keeps every
-// off-diagonal product below 2^30, so that it converts with a 32-bit
+// at most hbound x 2 max(|Re psi|, |Im psi|) -- stays below 2^62 (in split form
+// 2^46, see fx_put): no partial sum can overflow.  For complex64, F also keeps
+// every off-diagonal product below 2^30, so that it converts with a 32-bit
 // instruction; its rounding,
 // at most 2^-(F+1), is then about 1e-9 of the largest possible product, and
 // an entry of H psi collects it from at most a few thousand products.  For
@@ -595,9 +595,10 @@ __global__ void __launch_bounds__(kSpThreads, 1) k_apply_h_sparse(const SparseAr
   const bool base_smem = a.base_smem;
   for (uint32_t j = threadIdx.x; j < kAccBytes / 16u; j += NT)
     reinterpret_cast<uint4*>(acc)[j] = make_uint4(0u, 0u, 0u, 0u);
-  // fixed-point scale 2^F: every sum below 2^62 (complex64: 2^46), hbound x
-  // 2 max|component| x 2^F, and, for complex64, every off-diagonal product
-  // below 2^30 (dmax x 2 max|component| x 2^F <= 2^30)
+  // fixed-point scale 2^F: every sum below 2^62 (split: 2^46, which binds for
+  // no H that takes the split form), hbound x 2 max|component| x 2^F, and, for
+  // complex64, every off-diagonal product below 2^30 (dmax x 2 max|component| x
+  // 2^F <= 2^30)
   int F = 0;
   {
     const double m = __longlong_as_double((long long)*a.amax);
@@ -605,7 +606,7 @@ __global__ void __launch_bounds__(kSpThreads, 1) k_apply_h_sparse(const SparseAr
     if (bnd > 0.0) {
       int e;
       frexp(bnd, &e);   // bnd < 2^e
-      F = (sizeof(R) == 4 ? 46 : 62) - e;
+      F = (SPLIT ? 46 : 62) - e;
       if (sizeof(R) == 4 && bnd1 > 0.0) {
         frexp(bnd1, &e);
         F = min(F, 30 - e);
@@ -933,10 +934,12 @@ int sparse_apply_h(SparseArgs<R> a, const LiveOctets& lv, int sm_count, cudaStre
   a.toff = lv.toff;
   // complex64 adds its products in split form when every accumulator word
   // takes fewer than 65536 of them (at most one per off-diagonal group and
-  // diagonal piece); the two
-  // forms give the same integers, so H psi does not depend on the choice
+  // diagonal piece), and hbound is at most 2^15 times the largest weight, so
+  // that totals below 2^46 cost the products no bits (a large constant beside
+  // small couplings takes the carry form, whose totals have 62); the two
+  // forms then give the same integers, so H psi does not depend on the choice
   // (GOCP_SCATTER_SPLIT=0 selects the carry form)
-  bool split = sizeof(R) == 4 && a.n_offdiag + (uint32_t)a.sp.n_pieces < 65536u;
+  bool split = sizeof(R) == 4 && a.n_offdiag + (uint32_t)a.sp.n_pieces < 65536u && a.hbound <= 0x1p15 * a.dmax;
   if (const char* ev = std::getenv("GOCP_SCATTER_SPLIT"))
     if (ev[0] == '0') split = false;
   auto kern = split ? k_apply_h_sparse<R, sizeof(R) == 4> : k_apply_h_sparse<R, false>;

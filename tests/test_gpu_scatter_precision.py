@@ -71,3 +71,30 @@ def test_small_term_group_keeps_its_weights(n, small, monkeypatch):
     F = _scale(sum(sums), max(sums), m)
     tol = 2.0 ** -(F + 1) + m * sums[1] * (2.0 ** -22 + len(groups[1][1]) * 2.0 ** -30)
     assert np.max(np.abs(got[only] - ref[only])) <= tol
+
+
+def test_large_constant_leaves_the_products_their_precision(monkeypatch):
+    """A constant 2^30 times the largest off-diagonal weight: outputs without an
+    amplitude of their own are held to half a unit of 2^F per product."""
+    monkeypatch.setenv("GOCP_SPARSE_FRAC", "0.25")
+    n, m = 15, 0.05
+    rng = np.random.default_rng(3)
+    groups = []
+    for gx in (5, 6, 1 << (n - 1)):
+        zc = int(rng.integers(0, 1 << n))
+        zs = [zc ^ y for y in [0] + [1 << q for q in range(n)]]
+        groups.append((gx, zs, rng.normal(size=len(zs))))
+    groups.append((9, [3], [0.7]))          # a LUT group
+    sums = [float(np.sum(np.abs(w))) for _, _, w in groups]
+    H, p = _problem(n, groups, diagonal=[(0, 2.0 ** 30 * max(sums)), (7, 1.5)])
+    at = rng.permutation(1 << n)[:400]
+    psi = np.zeros(1 << n, np.complex128)
+    psi[at] = float(np.float32(m)) * rng.choice([-1.0, 1.0], size=at.size)
+    got, ref = _run(p, psi), sv.apply_terms(H, psi)
+    off = np.setdiff1d(np.concatenate([at ^ g[0] for g in groups]), at)
+    F = _scale(2.0 ** 30 * max(sums) + 1.5 + sum(sums), max(sums), m)
+    tol = len(groups) * (2.0 ** -(F + 1) + m * max(sums) * (2.0 ** -22 + n * 2.0 ** -30))
+    assert F == 30 - math.frexp(2.0 * max(sums) * m)[1]
+    assert np.max(np.abs(got[off] - ref[off])) <= tol
+    own = np.abs(got[at] - ref[at]) / np.abs(ref[at])
+    assert np.max(own) <= 2.0 ** -22
