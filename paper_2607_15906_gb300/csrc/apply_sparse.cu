@@ -358,6 +358,10 @@ __device__ __forceinline__ long long q_mul(long long a, long long b) {
   return (long long)((hi << 1) + (lo >> 63) + ((lo >> 62) & 1ull));
 }
 
+// Not a number, or infinite (on the bits).
+__device__ __forceinline__ bool not_finite(float v) { return (__float_as_uint(v) & 0x7F800000u) == 0x7F800000u; }
+__device__ __forceinline__ bool not_finite(double v) { return (__double2hiint(v) & 0x7FF00000) == 0x7FF00000; }
+
 // The lane's amplitude in the form its products take: scaled by 2^F
 // (complex64), or as v_q (complex128, see q_mul).
 template <typename R> struct SpVal;
@@ -820,11 +824,14 @@ __global__ void __launch_bounds__(kSpThreads, 1) k_apply_h_sparse(const SparseAr
     // epilogue, first the energy partials over the nonzero amplitudes of the
     // own tile (zero amplitudes add nothing): one full warp of amplitudes at a
     // time, since the FP64 pipe is narrow here
+    bool bad = false;   // an amplitude that fixed point cannot hold
+    const uint32_t e0 = a.toff[t], e1 = a.toff[t + 1];
     {
       double2 w = make_double2(0.0, 0.0);   // this thread's |psi|^2 and Re<psi|H psi> partials
-      const uint32_t e0 = a.toff[t], e1 = a.partials ? a.toff[t + 1] : e0;
       for (uint32_t e = e0 + threadIdx.x; e < e1; e += NT) {
         const C_t<R> q = a.aval[e];
+        bad = bad || not_finite(q.x) || not_finite(q.y);
+        if (!a.partials) continue;
         const uint32_t at = 4u * (a.aidx[e] & (kSpTile - 1u));
         w.x += (double)q.x * q.x;
         w.y += (double)q.x * ((double)acc_get(acc, at + kRe) * dn);
@@ -844,7 +851,7 @@ __global__ void __launch_bounds__(kSpThreads, 1) k_apply_h_sparse(const SparseAr
         }
       }
     }
-    __syncthreads();
+    const bool bad_tile = __syncthreads_or(bad);
     if (a.partials && warp < 2) {
       const double sum = warp_sum(s_red[warp][lane]);
       if (lane == 0) a.partials[2u * t + warp] = sum;
@@ -886,6 +893,12 @@ __global__ void __launch_bounds__(kSpThreads, 1) k_apply_h_sparse(const SparseAr
       }
     }
     __syncthreads();
+    if (bad_tile)   // what is not finite shows at its own entry, as in a floating-point diagonal
+      for (uint32_t e = e0 + threadIdx.x; e < e1; e += NT) {
+        const C_t<R> q = a.aval[e];
+        const R v = (q.x - q.x) + (q.y - q.y);
+        if (not_finite(v)) a.out[a.aidx[e]] = cmake<R>(v, v);
+      }
   }
   if (!a.partials) return;
   // the last block to finish adds the per-tile partials in tile order, so E
