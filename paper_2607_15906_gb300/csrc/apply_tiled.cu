@@ -306,8 +306,6 @@ __global__ void __launch_bounds__(256) k_octet_mask(const C_t<R>* __restrict__ p
   }
 }
 
-constexpr int kTiledParts = 16;
-
 // Bit t of flags (zeroed before) = tile t, 2^shift mask words, holds a marked
 // octet; *tile_counter = 0.
 __global__ void __launch_bounds__(256) k_mask_flags(const uint32_t* __restrict__ mask, uint32_t words, int shift,

@@ -671,6 +671,8 @@ int tiled_apply_h(const DevTables& t, const LiveOctets& lv, int precision, int s
 // Whether a tiled_apply_h call lists psi's nonzero amplitudes into lv.
 bool scatter_lists(const DevTables& t, const LiveOctets& lv);
 
+constexpr int kTiledParts = 16;   // blocks that share a tile of the staged kernel, at most
+
 // Pieces the scatter kernel takes (four bytes of shared memory each); a
 // problem with more keeps every state on the staged kernel.
 constexpr int kSpMaxPieces = 8192;

@@ -51,9 +51,10 @@ constexpr int kItemBlocksPerSm = 2;  // batched stages: blocks per item per SM
 // List chains (k_chain_list).
 constexpr uint64_t kListMaxAny = 65536, kListClusterC64 = 8192, kListClusterC128 = 2048;   // list_chain_blocks
 constexpr int kListMaxBlocks = 256;
-// Entries of the list and inbox buffers: a quarter of the state, 65,536 at
-// least (the inboxes of small states need room beyond their even share).
-uint32_t list_room(int n) { return std::max(1u << (n - 2), 65536u); }
+// Entries of the list and inbox buffers: a quarter of the state; for small
+// states, whose inboxes need room beyond their even share, twice the state up to
+// 65,536.
+uint32_t list_room(int n) { return std::max(1u << (n - 2), std::min(2u << n, 65536u)); }
 
 struct DeviceTables {
   DevTables t;
@@ -2522,8 +2523,11 @@ int build_tiled(int n, const std::vector<HLut<R>>& hl, const std::vector<uint32_
   // few output tiles (below 512: up to 21 qubits): global accumulators for
   // the scatter kernel's blocks that share a tile, zero between calls
   if (ntiles < 512) {
-    // (8 MiB at least: the staged kernel's parts of a small state go there too)
-    const size_t words = std::max(ntiles * (size_t)kSpTile * 2u, (size_t)1 << 20);
+    // (the sums of the staged kernel's parts go there too: as many as its pieces
+    // allow, up to 8 MiB)
+    const size_t parts = std::min<size_t>(kTiledParts, pieces.size()) - 1;
+    const size_t words = std::max(ntiles * (size_t)kSpTile * 2u,
+                                  std::min((parts * sizeof(C_t<R>) << n) / sizeof(unsigned long long), (size_t)1 << 20));
     if ((rc = dalloc(d, &d.live.gacc, words, bytes)) || (rc = dalloc(d, &d.live.tdone, ntiles, bytes))) return rc;
     if ((rc = cuda_status(cudaMemset(d.live.gacc, 0, words * sizeof(unsigned long long)), "zero gacc")) ||
         (rc = cuda_status(cudaMemset(d.live.tdone, 0, ntiles * sizeof(unsigned int)), "zero tdone")))
