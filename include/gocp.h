@@ -196,20 +196,25 @@ int gocp_reference_state(const gocp_problem* p, void* psi, void* stream);
  * psi' = sum_{m=0..5} theta^m/m! v_m (Eq. 5).  ops/theta are host or device
  * arrays per `mem`; ops must lie in [0, pool_size) (GOCP_EINVAL for host
  * arrays; device arrays are clamped and flagged, see gocp_device_errors).
- * n_ops may be 0.  A chain of several steps on a full-layout state of at
- * most 128 KiB (complex128: 11 qubits) runs in one thread block over shared
- * memory; a chain on a larger state whose nonzero amplitudes are bounded (a
- * problem built from integrals: the reference's determinants) runs in one
- * launch whose blocks walk the list of nonzero amplitudes and wait for one
- * another between steps (one cluster of 16 for short lists, every SM for longer
- * ones; such a wait gives up after 2 s, or GOCP_CHAIN_WAIT_NS nanoseconds when
- * that environment variable is set, see gocp_device_errors); other chains run
- * one launch per step, replayed as a CUDA graph whose steps are joined by
- * programmatic dependencies (GOCP_CHAIN_PDL=0: by full completion).  The
- * environment variable GOCP_ONCHIP_CHAINS selects other forms: "off" a launch
- * per step, "block" the one-block form where it fits, else that, "all" also a
- * cluster's shared memory for states up to 2 MiB, "list" the list form
- * for every problem (GOCP_LIST_SHARE caps the entries a block of it keeps in
+ * n_ops may be 0.  How a chain of several steps runs:
+ *  - on a full-layout state of at most 128 KiB (complex128: 11 qubits), in one
+ *    thread block over shared memory;
+ *  - on a larger state whose nonzero amplitudes are bounded (a problem built
+ *    from integrals: the reference's determinants; one given as tables up to 16
+ *    qubits), in one launch whose blocks walk the list of nonzero amplitudes and
+ *    wait for one another between steps: one cluster of 16 for short lists, with
+ *    its hardware barrier, which has no limit, and every SM for longer ones, with
+ *    a wait that gives up after 2 s, or GOCP_CHAIN_WAIT_NS nanoseconds when that
+ *    environment variable is set, see gocp_device_errors;
+ *  - in the sector layout (8 qubits and more), in one launch over the pair lists
+ *    with the same limited wait;
+ *  - else one launch per step, replayed as a CUDA graph whose steps are joined by
+ *    programmatic dependencies (GOCP_CHAIN_PDL=0: by full completion).
+ * The environment variable GOCP_ONCHIP_CHAINS selects among them.  "off": a
+ * launch per step.  "block": one block where the state fits, and a launch per step
+ * otherwise.  "all": as "block", but in a cluster's shared memory for states of up
+ * to 2 MiB.  "list": the list form for every full-layout problem
+ * (GOCP_LIST_SHARE caps the entries a block of it keeps in
  * shared memory, GOCP_LIST_INBOX those that others may send it).  Where the
  * driver refuses a launch whose blocks wait for one another (GOCP_CHAIN_REFUSE=1:
  * as if it did), the chain takes a launch per step.  Every form gives the same

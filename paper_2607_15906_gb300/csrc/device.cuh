@@ -738,7 +738,7 @@ unsigned int* counters_ptr(Problem& p);
 int pool_finish(Problem& p, const double* part, int nbx, double* d_grads, cudaStream_t st);
 int ensure_stage(Problem& p, int n_ops);
 double* dpart_ptr(Problem& p);          // stage capacity x at least the SM count
-bool chain_forms_default();             // GOCP_ONCHIP_CHAINS is unset
+bool chain_in_one_launch();             // GOCP_ONCHIP_CHAINS is unset or "list"
 uint64_t chain_wait_ns();               // limit of a wait between the blocks of a chain
 constexpr int kChainRefused = 1;        // beside the GOCP_ codes: the chain's one launch was refused, nothing ran
 int launch_together(const cudaLaunchConfig_t& cfg, const void* kernel, void** args, bool* refused);

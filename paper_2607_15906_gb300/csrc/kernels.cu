@@ -3668,7 +3668,7 @@ uint64_t chain_wait_ns() {
   const long long v = std::atoll(e);
   return v < 0 ? kChainWaitNs : (uint64_t)v;
 }
-bool chain_forms_default() { return onchip_is(nullptr); }
+bool chain_in_one_launch() { return onchip_is(nullptr) || onchip_is("list"); }
 double* dpart_ptr(Problem& p) { return p.dev->dpart; }
 
 // d_dE[j] = the sum of dpart[j blocks .. (j + 1) blocks), in order.

@@ -682,12 +682,13 @@ int pair_grid(Problem& p, int per_sm) {
   return (int)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)sm_of(p) * per_sm));
 }
 
-// Blocks of a cooperative sector chain, 0: a launch per step (asked for by
-// GOCP_ONCHIP_CHAINS = "off", or no barrier word: below 8 qubits).  256 pairs of
+// Blocks of a cooperative sector chain, 0: a launch per step (asked for by a
+// value of GOCP_ONCHIP_CHAINS other than "list", or no barrier word: below 8
+// qubits).  256 pairs of
 // the longest list per block, at most every SM: with fewer the barrier costs
 // more than the shares save.
 int sec_chain_blocks(Problem& p, int n_ops) {
-  if (n_ops < 2 || !dev_tables(p).cl.sync || !chain_forms_default()) return 0;
+  if (n_ops < 2 || !dev_tables(p).cl.sync || !chain_in_one_launch()) return 0;
   return (int)std::max<int64_t>(1, std::min<int64_t>(sm_of(p), (p.sec->max_pairs + 255) / 256));
 }
 
