@@ -202,10 +202,11 @@ int gocp_reference_state(const gocp_problem* p, void* psi, void* stream);
  *  - on a larger state whose nonzero amplitudes are bounded (a problem built
  *    from integrals: the reference's determinants; one given as tables up to 16
  *    qubits), in one launch whose blocks walk the list of nonzero amplitudes and
- *    wait for one another between steps: one cluster of 16 for short lists, with
- *    its hardware barrier, which has no limit, and every SM for longer ones, with
- *    a wait that gives up after 2 s, or GOCP_CHAIN_WAIT_NS nanoseconds when that
- *    environment variable is set, see gocp_device_errors;
+ *    wait for one another between steps: one cluster of 16 for short lists (and
+ *    short chains, unless GOCP_CHAIN_WAIT_NS is set), with its hardware barrier,
+ *    which has no limit, and every SM for longer ones, with a wait that gives up
+ *    after 2 s, or GOCP_CHAIN_WAIT_NS nanoseconds when that environment variable is
+ *    set, see gocp_device_errors;
  *  - in the sector layout (8 qubits and more), in one launch over the pair lists
  *    with the same limited wait;
  *  - else one launch per step, replayed as a CUDA graph whose steps are joined by

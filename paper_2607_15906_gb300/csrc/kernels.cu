@@ -50,7 +50,7 @@ constexpr int kItemBlocksPerSm = 2;  // batched stages: blocks per item per SM
 
 // List chains (k_chain_list).
 constexpr uint64_t kListMaxAny = 65536, kListClusterC64 = 8192, kListClusterC128 = 2048;   // list_chain_blocks
-constexpr int kListMaxBlocks = 256;
+constexpr int kListMaxBlocks = 256, kListClusterOps = 24;
 // Entries of the list and inbox buffers: a quarter of the state; for small
 // states, whose inboxes need room beyond their even share, twice the state up to
 // 65,536.
@@ -3643,6 +3643,22 @@ uint64_t list_bound(const Problem& p, int n_ops, bool back) {
 // so a short list takes the cluster, whose barrier is cheaper, and a longer one
 // every SM (complex128 sooner: its FP64 work on the touched pairs).  101
 // operators at 24 qubits: forward 5.3 -> 3.8 us a step, backward 6.1 -> 4.3.
+//
+// The bound says little about a short forward chain from one determinant: 20
+// operators drawn from the pool reach some 200 to 500 amplitudes, 20 chosen to
+// reach as many as they can 1,200 to 5,000.  Up to kListClusterOps it takes the
+// cluster, whose launch also starts about 7 us sooner (not where
+// GOCP_CHAIN_WAIT_NS sets a limit, which the cluster's barrier does not keep).
+// Forward chain of a drawn
+// | spreading ansatz, us (launch per step, every SM, cluster):
+//   complex128 20q, 12 operators  51.4  51.7  44.3 |  53.5  55.5  47.3
+//                   24 operators 100.7  98.5  84.1 | 132.0 102.6  94.5
+//                   30 operators 131.4 121.7 103.1 | 186.3 127.0 152.3
+//   complex128 22q, 24 operators 115.1 103.4  94.5 | 145.9 109.6 111.8
+//   complex128 16q, 20 operators  79.5  80.1  67.9 |  87.4  86.2  71.9
+//   complex64  24q, 20 operators 106.2  89.5  82.9 | 110.5  93.6  85.9
+// From two operators on, both directions and layouts, no chain measured is slower
+// than a launch per step.
 template <typename R>
 int list_chain_blocks(const Problem& p, int n_ops, bool back) {
   const DeviceTables& d = *p.dev;
@@ -3653,7 +3669,9 @@ int list_chain_blocks(const Problem& p, int n_ops, bool back) {
   // a state that may fill: the enumerated pairs, on every SM's own launches
   if (!force && b == 1ull << p.n_qubits && b > kListMaxAny) return 0;
   if (smem_chain_optin<R>() != GOCP_OK) return 0;
-  if (b <= (sizeof(R) == 4 ? kListClusterC64 : kListClusterC128) &&
+  const char* limit = std::getenv("GOCP_CHAIN_WAIT_NS");
+  const bool brief = !back && n_ops <= kListClusterOps && b < 1ull << p.n_qubits && !(limit && *limit);
+  if ((brief || b <= (sizeof(R) == 4 ? kListClusterC64 : kListClusterC128)) &&
       cluster_fits(back ? (const void*)k_chain_list<R, true, true> : (const void*)k_chain_list<R, false, true>,
                    kClusterMax, list_smem<R>()))
     return kClusterMax;
