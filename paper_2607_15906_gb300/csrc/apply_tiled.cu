@@ -818,10 +818,10 @@ int launch_tiled(const DevTables& t, const LiveOctets& lv, int sm_count, const v
   // Fewer tiles than SMs: K blocks share a tile.  K (at most the room in
   // extra, kTiledParts and the pieces allow) makes the rounds of equal parts
   // over the SMs shortest; one more part has to shorten them by 4 % to pay for
-  // its pass.  Parts cut the pieces at equal shares of their bytes.  A dense
-  // state over 64 tiles, whose blocks left 88 of the 152 SMs idle: 4.44 -> 2.35
-  // ms (18 qubits complex128, K = 2), 247 -> 174 us (19-qubit all-pairs spin
-  // Hamiltonian, complex64, K = 3).
+  // its pass.  Parts cut the pieces at about equal shares of their bytes.  A dense
+  // state over 64 tiles, whose blocks left 88 of the 152 SMs idle: 4.44 -> 2.34
+  // ms (18 qubits complex128), 247 -> 174 us (19-qubit all-pairs spin
+  // Hamiltonian, complex64), both with K = 2.
   const uint64_t sms = (uint64_t)std::max(sm_count, 1);
   int K = 1;
   if (ntiles < sms && lv.gacc) {

@@ -654,7 +654,7 @@ int gocp_profile_read(int kind, int64_t* launches, double* total_ms) {
 
 const char* gocp_last_error(void) { return t_last_error.c_str(); }
 int64_t gocp_launch_count(void) { return g_launches.load(); }
-// The k_apply_h revision names the kernel that profiles/traffic.json was measured on.
-const char* gocp_version(void) { return "gocp-gb300 0.2 (sm_103a; k_apply_h_tiled=tiled-tma-r13; k_apply_h_sparse=scatter-cases-r19; chain=amp-list-ring-4; list=coop-list-1; onchip=smem-chain-3; sector=pair-lists-coop-2; chains=graphs-pdl-2; grads=nonzero-amps-2)"; }
+// The k_apply_h revision names the kernel that profiles/kernel_counters.json was measured on.
+const char* gocp_version(void) { return "gocp-gb300 0.2 (sm_103a; k_apply_h_tiled=tiled-tma-r13; k_apply_h_sparse=scatter-cases-r20; chain=amp-list-ring-4; list=coop-list-2; onchip=smem-chain-3; sector=pair-lists-coop-3; chains=graphs-pdl-2; grads=nonzero-amps-2)"; }
 
 }  // extern "C"
