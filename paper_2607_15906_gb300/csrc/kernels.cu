@@ -54,7 +54,7 @@ constexpr int kListMaxBlocks = 256, kListClusterOps = 24;
 // Entries of the list and inbox buffers: a quarter of the state; for small
 // states, whose inboxes need room beyond their even share, twice the state up to
 // 65,536.
-uint32_t list_room(int n) { return std::max(1u << (n - 2), std::min(2u << n, 65536u)); }
+uint32_t list_room(int n) { return std::max(1u << (n - 2), (uint32_t)std::min<uint64_t>(2ull << n, 65536ull)); }
 
 struct DeviceTables {
   DevTables t;
